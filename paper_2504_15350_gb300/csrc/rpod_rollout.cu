@@ -260,6 +260,312 @@ __global__ void __launch_bounds__(512, 1) k_rollout(RollArgs a) {
   }
 }
 
+// ---- pipelined rollout over a thread-block cluster ------------------------
+// Every prediction runs the whole window from zero states, but the windows of
+// consecutive predictions share all rows but one: when row r becomes known,
+// the T windows that contain it can all advance by one time step.  So instead
+// of T + L - 1 dependent phases per prediction there are L: layer 0 of all T
+// windows on row r, layer 1 on their new h_0, ..., then the head on the one
+// window that row r completes, which gives row r + 1.  The work per
+// prediction is the same (T steps of L cells), its dependent chain is T/L
+// times shorter, and a product has T columns instead of one.
+//
+// Samples never interact, so one cluster of CS CTAs owns one sample (clusters
+// beyond the GPU's capacity run later; nothing waits across clusters).  A CTA
+// owns U = ceil(H / CS) hidden units of every layer: their 4U gate rows of
+// W_x and W_h stay in shared memory, in the type the products read (half the
+// shared memory of widened copies for BF16, so 16 CTAs hold 2 x 256), and
+// multiply the cluster's h (k-major, the T windows' values contiguous) with
+// packed FP32 pairs of windows: a lane holds two gate rows x T sums, so an
+// inner step is one 4-byte weight load and T/4 broadcast 16-byte loads of h
+// for T packed FMAs.  New h values go to every CTA of the cluster by 16-byte
+// distributed-shared-memory stores, and the hardware cluster barrier ends the
+// phase; its wait overlaps the recurrent product of the next phase, which
+// needs only the previous row.  Every CTA computes the whole head itself (O x H
+// multiply-adds, about 0.2 us), which saves a third barrier per row.
+//
+// Bound: the FP32 pipes and the phase latency (product, partial sums over the
+// k-slices, gates, push, barrier).  2 x 256, window 10, 8 samples, 500 steps:
+// see the figure at rollout_pipelined.
+constexpr int kPipeWarps = 8;
+
+struct PipeArgs {
+  int I, H, L, O, T, d, U, CS, steps;
+  int LR, SUB, RB, SL;         // row lanes, k sub-slices per warp, row blocks, k-slices
+  const float* theta;
+  const void* w;               // weights in the products' type
+  int64_t off_w[4][3];
+  int64_t off_wy, off_by;
+  const float* window;         // B x T x I
+  float* out;                  // B x steps x O
+};
+
+__host__ __device__ inline int even_up(int x) { return (x + 1) & ~1; }
+
+// Shared memory of one CTA, in floats except the weights (element size ws).
+__host__ __device__ inline size_t pipe_smem_bytes(int I, int H, int L, int O, int U, int CS, int Tp,
+                                                  int SL, size_t ws) {
+  const size_t R = 4 * (size_t)U;
+  size_t w = 0;
+  for (int l = 0; l < L; ++l) w += R * (size_t)(even_up(l == 0 ? I : H) + even_up(H));
+  w += (size_t)O * H;
+  size_t f = (size_t)2 * L * even_up(CS * U) * Tp;  // h, two buffers per layer
+  f += (size_t)SL * R * (Tp + 1);                   // partial sums, and those of x W_x
+  f += (size_t)L * R + (size_t)L * U * Tp;          // biases, cell states
+  f += (size_t)even_up(I) + O;
+  return f * 4 + ((w * ws + 15) & ~(size_t)15) + 16;
+}
+
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 wpair(const __nv_bfloat16* p) {
+  return __bfloat1622float2(*(const __nv_bfloat162*)p);
+}
+__device__ __forceinline__ float2 wpair(const float* p) { return *(const float2*)p; }
+
+// acc += W(k, rows) h(k, windows) for k in [k0, k1) (k0 even, k1 - k0 even):
+// W k-major with R rows (this lane's two at W), h k-major with 2 NP windows.
+template <typename TW, int NP>
+__device__ __forceinline__ void pipe_prod(const TW* W, int R, const float* h, int k0, int k1,
+                                          uint64_t (&acc)[2][NP]) {
+#pragma unroll 4
+  for (int k = k0; k < k1; k += 2) {
+    const float2 wa = wpair(W + (size_t)k * R), wb = wpair(W + (size_t)(k + 1) * R);
+    const ulonglong2* hp = (const ulonglong2*)(h + (size_t)k * (2 * NP));
+    uint64_t hv[2 * NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const ulonglong2 v = hp[i];
+      hv[2 * i] = v.x;
+      hv[2 * i + 1] = v.y;
+    }
+    const uint64_t a0 = pack2(wa.x, wa.x), a1 = pack2(wa.y, wa.y);
+    const uint64_t b0 = pack2(wb.x, wb.x), b1 = pack2(wb.y, wb.y);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      acc[0][i] = fma2(a0, hv[i], acc[0][i]);
+      acc[1][i] = fma2(a1, hv[i], acc[1][i]);
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      acc[0][i] = fma2(b0, hv[NP + i], acc[0][i]);
+      acc[1][i] = fma2(b1, hv[NP + i], acc[1][i]);
+    }
+  }
+}
+
+template <typename TW, int NP>
+__global__ void __launch_bounds__(kPipeWarps * 32, 1) k_rollout_pipe(const __grid_constant__ PipeArgs a) {
+  namespace cg = cooperative_groups;
+  constexpr int Tp = 2 * NP;
+  constexpr int NT = kPipeWarps * 32;
+  extern __shared__ __align__(16) float sm[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int I = a.I, H = a.H, L = a.L, O = a.O, T = a.T, U = a.U, CS = a.CS;
+  const int rank = (int)cl.block_rank(), b = blockIdx.x / CS;
+  const int u0 = rank * U, R = 4 * U, Hr = even_up(CS * U);
+  const int Ip = even_up(I), Hp = even_up(H);
+  // ---- shared memory (16-byte pieces first: h, then the weights)
+  float* hs = sm;                                   // [L][2][Hr][Tp]
+  float* part = hs + (size_t)2 * L * Hr * Tp;       // [SL][R][Tp]
+  float* px = part + (size_t)a.SL * R * Tp;         // [SL][R]
+  float* bias = px + (size_t)a.SL * R;              // [L][R]
+  float* cst = bias + (size_t)L * R;                // [L][U][Tp]
+  float* xs = cst + (size_t)L * U * Tp;             // [Ip]
+  float* by = xs + Ip;                              // [O]
+  TW* wsm = (TW*)(sm + (((by + O - sm) + 3) & ~(ptrdiff_t)3));
+  const TW* W = (const TW*)a.w;
+  {
+    TW* p = wsm;
+    for (int l = 0; l < L; ++l) {
+      const int Il = l == 0 ? I : H, Ilp = even_up(Il);
+      for (int part_i = 0; part_i < 2; ++part_i) {  // W_x, then W_h
+        const int K = part_i ? H : Il, Kp = part_i ? Hp : Ilp;
+        const TW* src = W + a.off_w[l][part_i];
+        // read along k (contiguous), write k-major
+        for (int e = tid; e < R * Kp; e += NT) {
+          const int r = e / Kp, k = e % Kp, u = u0 + r % U;
+          p[(size_t)k * R + r] = (k < K && u < H) ? src[((int64_t)(r / U) * H + u) * K + k] : TW(0.f);
+        }
+        p += (size_t)R * Kp;
+      }
+      for (int r = tid; r < R; r += NT) {
+        const int u = u0 + r % U;
+        bias[l * R + r] = u < H ? a.theta[a.off_w[l][2] + (int64_t)(r / U) * H + u] : 0.f;
+      }
+    }
+    for (int e = tid; e < O * H; e += NT) p[e] = W[a.off_wy + e];
+    for (int e = tid; e < O; e += NT) by[e] = a.theta[a.off_by + e];
+    for (int e = tid; e < 2 * L * Hr * Tp; e += NT) hs[e] = 0.f;
+    for (int e = tid; e < L * U * Tp; e += NT) cst[e] = 0.f;
+    for (int e = tid; e < Ip; e += NT) xs[e] = 0.f;
+  }
+  // this lane's two gate rows and its k-slice
+  const int rb = warp % a.RB;
+  const int row = rb * 64 + 2 * (lane % a.LR);
+  const int slice = (warp / a.RB) * a.SUB + lane / a.LR;
+  const bool live = row < R;
+  auto span = [&](int Kp, int& k0, int& k1) {
+    const int c = 2 * ((Kp / 2 + a.SL - 1) / a.SL);
+    k0 = slice * c < Kp ? slice * c : Kp;
+    k1 = k0 + c < Kp ? k0 + c : Kp;
+  };
+  cl.sync();
+
+  const int rows = T + a.steps;  // the last one only takes the last prediction
+  for (int r = 0; r < rows; ++r) {
+    const int buf = r & 1, z = r % T;
+    const TW* wl = wsm;
+    for (int l = 0; l < L; ++l) {
+      const int Il = l == 0 ? I : H, Ilp = even_up(Il);
+      const TW* Wx = wl;
+      const TW* Wh = wl + (size_t)R * Ilp;
+      wl = Wh + (size_t)R * Hp;
+      float* hl = hs + (size_t)(2 * l) * Hr * Tp;
+      const bool last = r == rows - 1;
+      const bool pending = r > 0 || l > 0;
+      // a single layer's own h is what the pending barrier publishes
+      if (L == 1 && pending) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      uint64_t acc[2][NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) acc[0][i] = acc[1][i] = 0ull;
+      int k0, k1;
+      if (live && !last) {
+        span(Hp, k0, k1);
+        pipe_prod<TW, NP>(Wh + row, R, hl + (size_t)(buf ^ 1) * Hr * Tp, k0, k1, acc);
+        // the window that starts with this row starts from h = 0
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            float v0, v1;
+            unpack2(acc[q][i], v0, v1);
+            acc[q][i] = pack2(2 * i == z ? 0.f : v0, 2 * i + 1 == z ? 0.f : v1);
+          }
+      }
+      if (L > 1 && pending) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      if (l == 0) {
+        // row r of the sequence: the given window, then the predictions (the
+        // parameters of the newest given row carry over)
+        if (r < T) {
+          for (int k = tid; k < I; k += NT) xs[k] = a.window[((int64_t)b * T + r) * I + k];
+        } else {
+          const float* ht = hs + (size_t)(2 * (L - 1) + (buf ^ 1)) * Hr * Tp + z;
+          const TW* Wy = wsm;
+          for (int l2 = 0; l2 < L; ++l2) Wy += (size_t)R * (even_up(l2 == 0 ? I : H) + Hp);
+          // eight outputs per warp at a time, lanes over k, then a transposing
+          // butterfly: lane group (lane >> 2) ends with output j = bits 4, 3, 2
+          for (int o0 = warp; o0 < O; o0 += 8 * kPipeWarps) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = 0.f;
+            for (int k = lane; k < H; k += 32) {
+              const float hv = ht[(size_t)k * Tp];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const int o = o0 + j * kPipeWarps;
+                if (o < O) v[j] = fmaf(wld(Wy + (size_t)o * H + k), hv, v[j]);
+              }
+            }
+#pragma unroll
+            for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1)
+#pragma unroll
+              for (int i = 0; i < n; ++i) {
+                const bool up = (lane & m) != 0;
+                const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + n], m);
+                v[i] = (up ? v[i + n] : v[i]) + got;
+              }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+            const int o = o0 + j * kPipeWarps;
+            if ((lane & 3) == 0 && o < O) {
+              const float y = v[0] + by[o];
+              xs[a.d + o] = y;
+              if (o % CS == rank) a.out[((int64_t)b * a.steps + (r - T)) * O + o] = y;
+            }
+          }
+        }
+        if (last) return;
+        __syncthreads();
+        if (live) {
+          span(Ip, k0, k1);
+          float x0 = 0.f, x1 = 0.f;
+          for (int k = k0; k < k1; ++k) {
+            const float2 w = wpair(Wx + (size_t)k * R + row);
+            x0 = fmaf(w.x, xs[k], x0);
+            x1 = fmaf(w.y, xs[k], x1);
+          }
+          px[slice * R + row] = x0;
+          px[slice * R + row + 1] = x1;
+        }
+      } else if (live) {
+        span(Ilp, k0, k1);
+        pipe_prod<TW, NP>(Wx + row, R, hs + (size_t)(2 * (l - 1) + buf) * Hr * Tp, k0, k1, acc);
+      }
+      if (live) {
+        uint64_t* d0 = (uint64_t*)(part + ((size_t)slice * R + row) * Tp);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          d0[i] = acc[0][i];
+          d0[NP + i] = acc[1][i];
+        }
+      }
+      __syncthreads();
+      // gates and cell update of this CTA's units
+      float* hnew = hl + (size_t)buf * Hr * Tp + (size_t)u0 * Tp;
+      for (int e = tid; e < U * Tp; e += NT) {
+        const int u = e / Tp, w = e % Tp;
+        float g[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) g[q] = bias[l * R + q * U + u];
+        for (int s = 0; s < a.SL; ++s)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) g[q] += part[((size_t)s * R + q * U + u) * Tp + w];
+        if (l == 0)
+          for (int s = 0; s < a.SL; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) g[q] += px[s * R + q * U + u];
+        float* cp = cst + (size_t)l * U * Tp + e;
+        const float c = sigm_r(g[1]) * (w == z ? 0.f : *cp) + sigm_r(g[0]) * tanhf(g[2]);
+        *cp = c;
+        hnew[e] = sigm_r(g[3]) * tanhf(c);
+      }
+      __syncthreads();
+      // this CTA's block of h to every other CTA of the cluster
+      const int n4 = U * Tp / 4, n2 = (U * Tp - 4 * n4) / 2;  // Tp is even
+      for (int e = tid; e < (CS - 1) * n4; e += NT) {
+        const int dst = (rank + 1 + e / n4) % CS, i = e % n4;
+        float* rem = cl.map_shared_rank(hnew, dst);
+        if (((U * Tp) & 3) == 0)
+          ((float4*)rem)[i] = ((const float4*)hnew)[i];
+        else {  // u0 Tp is a multiple of 2 only
+          ((float2*)rem)[2 * i] = ((const float2*)hnew)[2 * i];
+          ((float2*)rem)[2 * i + 1] = ((const float2*)hnew)[2 * i + 1];
+        }
+      }
+      if (n2)
+        for (int e = tid; e < CS - 1; e += NT) {
+          float* rem = cl.map_shared_rank(hnew, (rank + 1 + e) % CS);
+          ((float2*)rem)[2 * n4] = ((const float2*)hnew)[2 * n4];
+        }
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    }
+  }
+}
+
 // Self-test of the grid barrier's limit: CTA 0 never arrives, so the wait
 // of every CTA runs out and records the timeout.  Its words live here (the
 // library allocates nothing): [0] arrivals, [1] abort word, [2] status.
@@ -318,6 +624,99 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((void*)k_rollout<float>, grid, block, args, smem, st);
   }
   note_launch();
+  return e;
+}
+
+namespace {
+
+template <typename TW, int NP>
+cudaError_t launch_pipe(cudaStream_t st, PipeArgs& a, int B, size_t smem) {
+  auto fn = k_rollout_pipe<TW, NP>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && a.CS > 8)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(B * a.CS));
+  cfg.blockDim = dim3(kPipeWarps * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)a.CS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  // a cluster that the device cannot hold at all is refused here, before
+  // anything is enqueued
+  int active = 0;
+  e = cudaOccupancyMaxActiveClusters(&active, fn, &cfg);
+  if (e != cudaSuccess || active < 1) {
+    cudaGetLastError();
+    return cudaErrorInvalidConfiguration;
+  }
+  return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
+template <typename TW>
+cudaError_t launch_pipe_np(cudaStream_t st, PipeArgs& a, int B, int np, size_t smem) {
+  switch (np) {
+    case 2: return launch_pipe<TW, 2>(st, a, B, smem);
+    case 4: return launch_pipe<TW, 4>(st, a, B, smem);
+    case 5: return launch_pipe<TW, 5>(st, a, B, smem);
+    case 6: return launch_pipe<TW, 6>(st, a, B, smem);
+    default: return launch_pipe<TW, 8>(st, a, B, smem);
+  }
+}
+
+}  // namespace
+
+cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,
+                              int B, int d, int steps, const float* theta, const void* wbf,
+                              const int64_t (*off_w)[3], int64_t off_wy, int64_t off_by,
+                              const float* window, float* out, int sms) {
+  if (L > 4 || T > 16) return cudaErrorInvalidConfiguration;
+  const int np = T <= 4 ? 2 : (T <= 8 ? 4 : (T <= 10 ? 5 : (T <= 12 ? 6 : 8)));
+  const size_t wsz = bf16_weights ? 2 : 4;
+  PipeArgs a;
+  a.I = I; a.H = H; a.L = L; a.O = O; a.T = T; a.d = d; a.steps = steps;
+  a.theta = theta;
+  a.w = wbf;
+  for (int l = 0; l < L; ++l)
+    for (int j = 0; j < 3; ++j) a.off_w[l][j] = off_w[l][j];
+  a.off_wy = off_wy;
+  a.off_by = off_by;
+  a.window = window;
+  a.out = out;
+  // the largest cluster that leaves a CTA four units and lets the samples'
+  // clusters run in at most two waves; if none does, the smallest whose CTAs
+  // hold their weights
+  int pick = 0;
+  auto shape = [&](int CS) {
+    a.CS = CS;
+    a.U = (H + CS - 1) / CS;
+    const int R = 4 * a.U;
+    a.LR = 1;
+    while (a.LR < 32 && 2 * a.LR < R) a.LR <<= 1;
+    a.SUB = 32 / a.LR;
+    a.RB = 1;
+    while (64 * a.RB < R) a.RB <<= 1;
+    if (a.RB > kPipeWarps) return (size_t)-1;
+    a.SL = kPipeWarps / a.RB * a.SUB;
+    return pipe_smem_bytes(I, H, L, O, a.U, CS, 2 * np, a.SL, wsz);
+  };
+  for (int CS = 16; CS >= 1; CS >>= 1) {
+    if (CS > 1 && (H + CS - 1) / CS < 4) continue;
+    if (shape(CS) > (size_t)227 * 1024) break;
+    pick = CS;
+    if ((int64_t)B * CS <= 2 * sms) break;
+  }
+  if (!pick) return cudaErrorInvalidConfiguration;
+  const size_t smem = shape(pick);
+  const cudaError_t e = bf16_weights ? launch_pipe_np<__nv_bfloat16>(st, a, B, np, smem)
+                                     : launch_pipe_np<float>(st, a, B, np, smem);
+  if (e == cudaSuccess) note_launch();
   return e;
 }
 
