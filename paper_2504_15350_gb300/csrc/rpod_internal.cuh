@@ -206,7 +206,7 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
 cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,
                               int B, int d, int steps, const float* theta, const void* wbf,
                               const int64_t (*off_w)[3], int64_t off_wy, int64_t off_by,
-                              const float* window, float* out, int sms);
+                              const float* window, float* out, unsigned* status);
 cudaError_t grid_sync_selftest(cudaStream_t st, double seconds, unsigned* status_out);
 
 // Sets every kernel attribute the library needs (dynamic shared memory

@@ -641,17 +641,13 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
   cudaStream_t st = (cudaStream_t)stream;
   Net net{N, (char*)ws, st};
   g_launches = 0;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return RPOD_ERR_CUDA;
   unsigned* sync = (unsigned*)((char*)ws + N->o_sync);
   LK(cudaMemsetAsync(sync, 0, 16, st));  // barrier arrivals, abort word, status word
   {
     const cudaError_t e = rollout_pipelined(
         st, !N->wfp32, N->I, N->H, N->L, N->O, N->T, B, mu_cols, steps, net.f(N->o_theta),
         N->wfp32 ? (const void*)net.f(N->o_theta) : (const void*)net.wbf(), N->off_w, N->off_wy,
-        N->off_by, window, out, sms);
+        N->off_by, window, out, sync + 2);
     if (e == cudaSuccess) {
       N->last_launches = g_launches;
       return RPOD_OK;
@@ -662,6 +658,10 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
   float* nxt = net.f(N->o_xtm2);
   k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, window, cur);
   LL();
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return RPOD_ERR_CUDA;
   if (rollout_fits(N, B, sms)) {
     // one cooperative launch for all steps (the window in o_xtm is its ring)
     const cudaError_t e = rollout_persistent(

@@ -19,6 +19,8 @@
 // kernel returns; nothing waits without a limit.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "rpod_internal.cuh"
 
 namespace rpod {
@@ -267,53 +269,54 @@ __global__ void __launch_bounds__(512, 1) k_rollout(RollArgs a) {
 // of T + L - 1 dependent phases per prediction there are L: layer 0 of all T
 // windows on row r, layer 1 on their new h_0, ..., then the head on the one
 // window that row r completes, which gives row r + 1.  The work per
-// prediction is the same (T steps of L cells), its dependent chain is T/L
-// times shorter, and a product has T columns instead of one.
+// prediction is the same (T steps of L cells), its dependent chain is T times
+// shorter, and a product has T columns instead of one.
 //
 // Samples never interact, so one cluster of CS CTAs owns one sample (clusters
 // beyond the GPU's capacity run later; nothing waits across clusters).  A CTA
-// owns U = ceil(H / CS) hidden units of every layer: their 4U gate rows of
-// W_x and W_h stay in shared memory, in the type the products read (half the
-// shared memory of widened copies for BF16, so 16 CTAs hold 2 x 256), and
-// multiply the cluster's h (k-major, the T windows' values contiguous) with
-// packed FP32 pairs of windows: a lane holds two gate rows x T sums, so an
-// inner step is one 4-byte weight load and T/4 broadcast 16-byte loads of h
-// for T packed FMAs.  New h values go to every CTA of the cluster by 16-byte
-// distributed-shared-memory stores, and the hardware cluster barrier ends the
-// phase; its wait overlaps the recurrent product of the next phase, which
-// needs only the previous row.  Every CTA computes the whole head itself (O x H
-// multiply-adds, about 0.2 us), which saves a third barrier per row.
+// owns U hidden units of every layer: their 4U gate rows of W_x and W_h stay
+// in shared memory, in the type the products read (half the shared memory of
+// widened copies for BF16), and multiply the cluster's h (k-major, the T
+// windows' values contiguous) with packed FP32 pairs of windows: a thread
+// holds two gate rows x T sums of one k-slice, so an inner step is one 4-byte
+// weight load and T/4 broadcast 16-byte loads of h for T packed FMAs.  New h
+// values go to every CTA of the cluster as bulk copies between shared memories
+// that complete on the receiver's mbarrier; the wait for them comes after the
+// next phase's recurrent product, which needs only the previous row.  The head is split over the units: each CTA sends its share of
+// the O outputs with its h, and every CTA adds the CS shares itself.
 //
-// Bound: the FP32 pipes and the phase latency (product, partial sums over the
-// k-slices, gates, push, barrier).  2 x 256, window 10, 8 samples, 500 steps:
-// see the figure at rollout_pipelined.
-constexpr int kPipeWarps = 8;
+// Bound: the FP32 pipes (3 products of 4U x T x H per row and CTA) and the
+// phase latency (partial sums over the k-slices, gates, exchange).  Measured
+// at 2 x 256, window 10, 8 samples, 500 steps: 4.1 ms; the kernel with
+// T + L - 1 grid barriers per prediction above takes 68.4 ms.
+constexpr int kPipeThreads = 384;
 
 struct PipeArgs {
   int I, H, L, O, T, d, U, CS, steps;
-  int LR, SUB, RB, SL;         // row lanes, k sub-slices per warp, row blocks, k-slices
+  int SL, threads;             // k-slices, threads that multiply (SL x 2U)
   const float* theta;
   const void* w;               // weights in the products' type
   int64_t off_w[4][3];
   int64_t off_wy, off_by;
   const float* window;         // B x T x I
   float* out;                  // B x steps x O
+  unsigned* status;
 };
 
 __host__ __device__ inline int even_up(int x) { return (x + 1) & ~1; }
 
-// Shared memory of one CTA, in floats except the weights (element size ws).
+// Shared memory of one CTA; ws: bytes of a stored weight.
 __host__ __device__ inline size_t pipe_smem_bytes(int I, int H, int L, int O, int U, int CS, int Tp,
                                                   int SL, size_t ws) {
   const size_t R = 4 * (size_t)U;
-  size_t w = 0;
+  size_t w = (size_t)O * U;
   for (int l = 0; l < L; ++l) w += R * (size_t)(even_up(l == 0 ? I : H) + even_up(H));
-  w += (size_t)O * H;
-  size_t f = (size_t)2 * L * even_up(CS * U) * Tp;  // h, two buffers per layer
-  f += (size_t)SL * R * (Tp + 1);                   // partial sums, and those of x W_x
-  f += (size_t)L * R + (size_t)L * U * Tp;          // biases, cell states
+  size_t f = (size_t)2 * L * CS * U * Tp;        // h, two buffers per layer
+  f += (size_t)2 * CS * ((O + 3) & ~3);          // head shares
+  f += (size_t)SL * R * Tp;                      // partial sums
+  f += (size_t)L * R + (size_t)L * U * Tp;       // biases, cell states
   f += (size_t)even_up(I) + O;
-  return f * 4 + ((w * ws + 15) & ~(size_t)15) + 16;
+  return f * 4 + ((w * ws + 15) & ~(size_t)15) + 64;
 }
 
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
@@ -329,20 +332,58 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ float2 wpair(const __nv_bfloat16* p) {
   return __bfloat1622float2(*(const __nv_bfloat162*)p);
 }
 __device__ __forceinline__ float2 wpair(const float* p) { return *(const float2*)p; }
 
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// bytes (a multiple of 16) from this CTA's shared memory to another's; the
+// writes were made visible to the async proxy before
+__device__ __forceinline__ void send_block(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t mbar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "r"(src), "r"(bytes), "r"(mbar)
+      : "memory");
+}
+// Bounded wait for a phase of the exchange; false when 2 s passed.
+__device__ __forceinline__ bool exch_wait(uint32_t mbar, uint32_t parity) {
+  uint32_t ok = 0;
+  const uint64_t t0 = gtimer();
+  while (true) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (gtimer() - t0 > kBarrierTimeoutNs) return false;
+  }
+}
+
 // acc += W(k, rows) h(k, windows) for k in [k0, k1) (k0 even, k1 - k0 even):
-// W k-major with R rows (this lane's two at W), h k-major with 2 NP windows.
+// W k-major with R rows (this thread's two at W), h k-major with 2 NP windows.
 template <typename TW, int NP>
 __device__ __forceinline__ void pipe_prod(const TW* W, int R, const float* h, int k0, int k1,
                                           uint64_t (&acc)[2][NP]) {
 #pragma unroll 4
   for (int k = k0; k < k1; k += 2) {
-    const float2 wa = wpair(W + (size_t)k * R), wb = wpair(W + (size_t)(k + 1) * R);
-    const ulonglong2* hp = (const ulonglong2*)(h + (size_t)k * (2 * NP));
+    const float2 wa = wpair(W + k * R), wb = wpair(W + (k + 1) * R);
+    const ulonglong2* hp = (const ulonglong2*)(h + k * (2 * NP));
     uint64_t hv[2 * NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -366,85 +407,104 @@ __device__ __forceinline__ void pipe_prod(const TW* W, int R, const float* h, in
 }
 
 template <typename TW, int NP>
-__global__ void __launch_bounds__(kPipeWarps * 32, 1) k_rollout_pipe(const __grid_constant__ PipeArgs a) {
+__global__ void __launch_bounds__(kPipeThreads, 1) k_rollout_pipe(const __grid_constant__ PipeArgs a) {
   namespace cg = cooperative_groups;
-  constexpr int Tp = 2 * NP;
-  constexpr int NT = kPipeWarps * 32;
+  constexpr int Tp = 2 * NP, NT = kPipeThreads;
   extern __shared__ __align__(16) float sm[];
+  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ volatile int s_dead;
   cg::cluster_group cl = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int I = a.I, H = a.H, L = a.L, O = a.O, T = a.T, U = a.U, CS = a.CS;
+  const int I = a.I, H = a.H, L = a.L, O = a.O, T = a.T, U = a.U, CS = a.CS, SL = a.SL;
   const int rank = (int)cl.block_rank(), b = blockIdx.x / CS;
-  const int u0 = rank * U, R = 4 * U, Hr = even_up(CS * U);
-  const int Ip = even_up(I), Hp = even_up(H);
-  // ---- shared memory (16-byte pieces first: h, then the weights)
+  const int u0 = rank * U, R = 4 * U, Hr = CS * U;
+  const int Ip = even_up(I), Hp = even_up(H), Op = (O + 3) & ~3;
+  // ---- shared memory (16-byte pieces first: h, head shares, weights)
   float* hs = sm;                                   // [L][2][Hr][Tp]
-  float* part = hs + (size_t)2 * L * Hr * Tp;       // [SL][R][Tp]
-  float* px = part + (size_t)a.SL * R * Tp;         // [SL][R]
-  float* bias = px + (size_t)a.SL * R;              // [L][R]
+  float* yp = hs + (size_t)2 * L * Hr * Tp;         // [2][CS][Op]
+  float* part = yp + (size_t)2 * CS * Op;           // [SL][R][Tp], gate row r = 4 u + gate
+  float* bias = part + (size_t)SL * R * Tp;         // [L][R]
   float* cst = bias + (size_t)L * R;                // [L][U][Tp]
   float* xs = cst + (size_t)L * U * Tp;             // [Ip]
   float* by = xs + Ip;                              // [O]
   TW* wsm = (TW*)(sm + (((by + O - sm) + 3) & ~(ptrdiff_t)3));
+  TW* wy;                                           // [O][U]
   const TW* W = (const TW*)a.w;
   {
     TW* p = wsm;
     for (int l = 0; l < L; ++l) {
       const int Il = l == 0 ? I : H, Ilp = even_up(Il);
-      for (int part_i = 0; part_i < 2; ++part_i) {  // W_x, then W_h
-        const int K = part_i ? H : Il, Kp = part_i ? Hp : Ilp;
-        const TW* src = W + a.off_w[l][part_i];
+      for (int pi = 0; pi < 2; ++pi) {  // W_x, then W_h
+        const int K = pi ? H : Il, Kp = pi ? Hp : Ilp;
+        const TW* src = W + a.off_w[l][pi];
         // read along k (contiguous), write k-major
         for (int e = tid; e < R * Kp; e += NT) {
-          const int r = e / Kp, k = e % Kp, u = u0 + r % U;
-          p[(size_t)k * R + r] = (k < K && u < H) ? src[((int64_t)(r / U) * H + u) * K + k] : TW(0.f);
+          const int r = e / Kp, k = e % Kp, u = u0 + (r >> 2);
+          p[k * R + r] = (k < K && u < H) ? src[((int64_t)(r & 3) * H + u) * K + k] : TW(0.f);
         }
         p += (size_t)R * Kp;
       }
       for (int r = tid; r < R; r += NT) {
-        const int u = u0 + r % U;
-        bias[l * R + r] = u < H ? a.theta[a.off_w[l][2] + (int64_t)(r / U) * H + u] : 0.f;
+        const int u = u0 + (r >> 2);
+        bias[l * R + r] = u < H ? a.theta[a.off_w[l][2] + (int64_t)(r & 3) * H + u] : 0.f;
       }
     }
-    for (int e = tid; e < O * H; e += NT) p[e] = W[a.off_wy + e];
+    wy = p;
+    for (int e = tid; e < O * U; e += NT) {
+      const int o = e / U, u = u0 + e % U;
+      wy[e] = u < H ? W[a.off_wy + (int64_t)o * H + u] : TW(0.f);
+    }
     for (int e = tid; e < O; e += NT) by[e] = a.theta[a.off_by + e];
     for (int e = tid; e < 2 * L * Hr * Tp; e += NT) hs[e] = 0.f;
     for (int e = tid; e < L * U * Tp; e += NT) cst[e] = 0.f;
     for (int e = tid; e < Ip; e += NT) xs[e] = 0.f;
   }
-  // this lane's two gate rows and its k-slice
-  const int rb = warp % a.RB;
-  const int row = rb * 64 + 2 * (lane % a.LR);
-  const int slice = (warp / a.RB) * a.SUB + lane / a.LR;
-  const bool live = row < R;
+  const uint32_t mb = smem_u32(mbar);
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb + 8 * i) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_dead = 0;
+  }
+  // this thread's two gate rows and its k-slice
+  const bool live = tid < a.threads;
+  const int slice = tid / (2 * U), row = 2 * (tid % (2 * U));
   auto span = [&](int Kp, int& k0, int& k1) {
-    const int c = 2 * ((Kp / 2 + a.SL - 1) / a.SL);
+    const int c = 2 * ((Kp / 2 + SL - 1) / SL);
     k0 = slice * c < Kp ? slice * c : Kp;
     k1 = k0 + c < Kp ? k0 + c : Kp;
   };
+  int hk0, hk1, xk0, xk1;
+  span(Hp, hk0, hk1);
+  span(Ip, xk0, xk1);
   cl.sync();
 
+  int g = 0;                     // exchanges started
   const int rows = T + a.steps;  // the last one only takes the last prediction
-  for (int r = 0; r < rows; ++r) {
+  bool dead = false;
+  for (int r = 0; r < rows && !dead; ++r) {
     const int buf = r & 1, z = r % T;
+    const bool last = r == rows - 1;
     const TW* wl = wsm;
     for (int l = 0; l < L; ++l) {
-      const int Il = l == 0 ? I : H, Ilp = even_up(Il);
+      const int Ilp = l == 0 ? Ip : Hp;
       const TW* Wx = wl;
       const TW* Wh = wl + (size_t)R * Ilp;
       wl = Wh + (size_t)R * Hp;
       float* hl = hs + (size_t)(2 * l) * Hr * Tp;
-      const bool last = r == rows - 1;
-      const bool pending = r > 0 || l > 0;
-      // a single layer's own h is what the pending barrier publishes
-      if (L == 1 && pending) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      auto arrived = [&]() {
+        if (g > 0 && !exch_wait(mb + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1)) {
+          atomicOr(a.status, ST_TIMEOUT);
+          s_dead = 1;
+        }
+      };
+      // a single layer's own h is what the exchange in flight brings
+      if (L == 1) arrived();
       uint64_t acc[2][NP];
 #pragma unroll
       for (int i = 0; i < NP; ++i) acc[0][i] = acc[1][i] = 0ull;
-      int k0, k1;
       if (live && !last) {
-        span(Hp, k0, k1);
-        pipe_prod<TW, NP>(Wh + row, R, hl + (size_t)(buf ^ 1) * Hr * Tp, k0, k1, acc);
+        pipe_prod<TW, NP>(Wh + row, R, hl + (size_t)(buf ^ 1) * Hr * Tp, hk0, hk1, acc);
         // the window that starts with this row starts from h = 0
 #pragma unroll
         for (int i = 0; i < NP; ++i)
@@ -455,68 +515,53 @@ __global__ void __launch_bounds__(kPipeWarps * 32, 1) k_rollout_pipe(const __gri
             acc[q][i] = pack2(2 * i == z ? 0.f : v0, 2 * i + 1 == z ? 0.f : v1);
           }
       }
-      if (L > 1 && pending) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      if (L > 1) arrived();
       if (l == 0) {
         // row r of the sequence: the given window, then the predictions (the
         // parameters of the newest given row carry over)
         if (r < T) {
           for (int k = tid; k < I; k += NT) xs[k] = a.window[((int64_t)b * T + r) * I + k];
         } else {
-          const float* ht = hs + (size_t)(2 * (L - 1) + (buf ^ 1)) * Hr * Tp + z;
-          const TW* Wy = wsm;
-          for (int l2 = 0; l2 < L; ++l2) Wy += (size_t)R * (even_up(l2 == 0 ? I : H) + Hp);
-          // eight outputs per warp at a time, lanes over k, then a transposing
-          // butterfly: lane group (lane >> 2) ends with output j = bits 4, 3, 2
-          for (int o0 = warp; o0 < O; o0 += 8 * kPipeWarps) {
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = 0.f;
-            for (int k = lane; k < H; k += 32) {
-              const float hv = ht[(size_t)k * Tp];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const int o = o0 + j * kPipeWarps;
-                if (o < O) v[j] = fmaf(wld(Wy + (size_t)o * H + k), hv, v[j]);
-              }
+          const float* ys = yp + (size_t)(buf ^ 1) * CS * Op;
+          for (int e0 = 0; e0 < 4 * Op; e0 += NT) {  // four lanes per output
+            const int e = e0 + tid, o = e >> 2;
+            float y = 0.f;
+            if (o < O) {
+#pragma unroll 4
+              for (int c = e & 3; c < CS; c += 4) y += ys[c * Op + o];
             }
-#pragma unroll
-            for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1)
-#pragma unroll
-              for (int i = 0; i < n; ++i) {
-                const bool up = (lane & m) != 0;
-                const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + n], m);
-                v[i] = (up ? v[i + n] : v[i]) + got;
-              }
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-            const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-            const int o = o0 + j * kPipeWarps;
-            if ((lane & 3) == 0 && o < O) {
-              const float y = v[0] + by[o];
+            y += __shfl_xor_sync(0xffffffffu, y, 1);
+            y += __shfl_xor_sync(0xffffffffu, y, 2);
+            if ((e & 3) == 0 && o < O) {
+              y += by[o];
               xs[a.d + o] = y;
-              if (o % CS == rank) a.out[((int64_t)b * a.steps + (r - T)) * O + o] = y;
+              if (rank == 0) a.out[((int64_t)b * a.steps + (r - T)) * O + o] = y;
             }
           }
         }
-        if (last) return;
+        if (last) break;
         __syncthreads();
         if (live) {
-          span(Ip, k0, k1);
+          // the row is the same for all windows
           float x0 = 0.f, x1 = 0.f;
-          for (int k = k0; k < k1; ++k) {
-            const float2 w = wpair(Wx + (size_t)k * R + row);
+#pragma unroll 4
+          for (int k = xk0; k < xk1; ++k) {
+            const float2 w = wpair(Wx + k * R + row);
             x0 = fmaf(w.x, xs[k], x0);
             x1 = fmaf(w.y, xs[k], x1);
           }
-          px[slice * R + row] = x0;
-          px[slice * R + row + 1] = x1;
+          const uint64_t p0 = pack2(x0, x0), p1 = pack2(x1, x1);
+#pragma unroll
+          for (int i = 0; i < NP; ++i) {
+            acc[0][i] = add2(acc[0][i], p0);
+            acc[1][i] = add2(acc[1][i], p1);
+          }
         }
       } else if (live) {
-        span(Ilp, k0, k1);
-        pipe_prod<TW, NP>(Wx + row, R, hs + (size_t)(2 * (l - 1) + buf) * Hr * Tp, k0, k1, acc);
+        pipe_prod<TW, NP>(Wx + row, R, hs + (size_t)(2 * (l - 1) + buf) * Hr * Tp, hk0, hk1, acc);
       }
       if (live) {
-        uint64_t* d0 = (uint64_t*)(part + ((size_t)slice * R + row) * Tp);
+        uint64_t* d0 = (uint64_t*)(part + (slice * R + row) * Tp);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
           d0[i] = acc[0][i];
@@ -524,46 +569,75 @@ __global__ void __launch_bounds__(kPipeWarps * 32, 1) k_rollout_pipe(const __gri
         }
       }
       __syncthreads();
-      // gates and cell update of this CTA's units
+      if (s_dead) {  // uniform: set before the barrier
+        dead = true;
+        break;
+      }
+      // sums over the k-slices, four values per thread, into the first slice
       float* hnew = hl + (size_t)buf * Hr * Tp + (size_t)u0 * Tp;
       for (int e = tid; e < U * Tp; e += NT) {
-        const int u = e / Tp, w = e % Tp;
-        float g[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) g[q] = bias[l * R + q * U + u];
-        for (int s = 0; s < a.SL; ++s)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) g[q] += part[((size_t)s * R + q * U + u) * Tp + w];
-        if (l == 0)
-          for (int s = 0; s < a.SL; ++s)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) g[q] += px[s * R + q * U + u];
-        float* cp = cst + (size_t)l * U * Tp + e;
-        const float c = sigm_r(g[1]) * (w == z ? 0.f : *cp) + sigm_r(g[0]) * tanhf(g[2]);
-        *cp = c;
-        hnew[e] = sigm_r(g[3]) * tanhf(c);
+        float4* p4 = (float4*)part + e;
+        float4 v = p4[0];
+#pragma unroll 8
+        for (int s = 1; s < SL; ++s) {
+          const float4 t = p4[s * U * Tp];
+          v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+        }
+        p4[0] = v;
       }
       __syncthreads();
-      // this CTA's block of h to every other CTA of the cluster
-      const int n4 = U * Tp / 4, n2 = (U * Tp - 4 * n4) / 2;  // Tp is even
-      for (int e = tid; e < (CS - 1) * n4; e += NT) {
-        const int dst = (rank + 1 + e / n4) % CS, i = e % n4;
-        float* rem = cl.map_shared_rank(hnew, dst);
-        if (((U * Tp) & 3) == 0)
-          ((float4*)rem)[i] = ((const float4*)hnew)[i];
-        else {  // u0 Tp is a multiple of 2 only
-          ((float2*)rem)[2 * i] = ((const float2*)hnew)[2 * i];
-          ((float2*)rem)[2 * i + 1] = ((const float2*)hnew)[2 * i + 1];
-        }
+      // gates and cell update of this CTA's units
+      for (int cell = tid; cell < U * Tp; cell += NT) {
+        const int u = cell / Tp, w = cell % Tp;
+        const float* ps = part + 4 * u * Tp + w;
+        const float* bs = bias + l * R + 4 * u;
+        const float gi = sigm_r(ps[0] + bs[0]), gf = sigm_r(ps[Tp] + bs[1]);
+        const float gg = tanhf(ps[2 * Tp] + bs[2]), go = sigm_r(ps[3 * Tp] + bs[3]);
+        float* cp = cst + l * U * Tp + cell;
+        const float c = gf * (w == z ? 0.f : *cp) + gi * gg;
+        *cp = c;
+        hnew[cell] = go * tanhf(c);
       }
-      if (n2)
-        for (int e = tid; e < CS - 1; e += NT) {
-          float* rem = cl.map_shared_rank(hnew, (rank + 1 + e) % CS);
-          ((float2*)rem)[2 * n4] = ((const float2*)hnew)[2 * n4];
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();
+      const uint32_t bar = mb + 8 * (g & 1);
+      const bool top = l == L - 1;
+      if (tid == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                     "r"((uint32_t)((CS - 1) * (U * Tp + (top ? Op : 0)) * 4))
+                     : "memory");
+      float* yo = yp + ((size_t)buf * CS + rank) * Op;
+      if (top) {
+        // this CTA's share of the head for the window that ends with row r,
+        // four lanes per output
+        const float* hw = hnew + (r + 1) % T;  // its slot
+        for (int e0 = 0; e0 < 4 * Op; e0 += NT) {
+          const int e = e0 + tid, o = e >> 2;
+          float v = 0.f;
+          if (o < O) {
+#pragma unroll 4
+            for (int u = e & 3; u < U; u += 4) v = fmaf(wld(wy + o * U + u), hw[u * Tp], v);
+          }
+          v += __shfl_xor_sync(0xffffffffu, v, 1);
+          v += __shfl_xor_sync(0xffffffffu, v, 2);
+          if ((e & 3) == 0 && o < Op) yo[o] = v;
         }
-      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+      }
+      // this CTA's block of h and head share to every other CTA of the cluster
+      // (bulk copies: per-lane asynchronous stores spent about 2000 clocks of
+      // the receivers' shared memory on mbarrier updates per phase)
+      for (int c = 1 + warp; c < CS && lane == 0; c += NT / 32) {
+        const int dst = rank + c < CS ? rank + c : rank + c - CS;
+        const uint32_t rbar = cluster_addr(bar, dst);
+        if (top) send_block(cluster_addr(smem_u32(yo), dst), smem_u32(yo), Op * 4, rbar);
+        send_block(cluster_addr(smem_u32(hnew), dst), smem_u32(hnew), U * Tp * 4, rbar);
+      }
+      ++g;
     }
   }
+  cl.sync();  // nothing is sent to a CTA that has left
 }
 
 // Self-test of the grid barrier's limit: CTA 0 never arrives, so the wait
@@ -629,8 +703,10 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
 
 namespace {
 
+// One cluster per sample: the launch, or with `active` only how many clusters
+// run at once (nothing enqueued).
 template <typename TW, int NP>
-cudaError_t launch_pipe(cudaStream_t st, PipeArgs& a, int B, size_t smem) {
+cudaError_t pipe_launch(cudaStream_t st, const PipeArgs& a, int B, size_t smem, int* active) {
   auto fn = k_rollout_pipe<TW, NP>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess && a.CS > 8)
@@ -638,7 +714,7 @@ cudaError_t launch_pipe(cudaStream_t st, PipeArgs& a, int B, size_t smem) {
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(B * a.CS));
-  cfg.blockDim = dim3(kPipeWarps * 32);
+  cfg.blockDim = dim3(kPipeThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -648,26 +724,29 @@ cudaError_t launch_pipe(cudaStream_t st, PipeArgs& a, int B, size_t smem) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  // a cluster that the device cannot hold at all is refused here, before
-  // anything is enqueued
-  int active = 0;
-  e = cudaOccupancyMaxActiveClusters(&active, fn, &cfg);
-  if (e != cudaSuccess || active < 1) {
-    cudaGetLastError();
-    return cudaErrorInvalidConfiguration;
-  }
+  if (active) return cudaOccupancyMaxActiveClusters(active, fn, &cfg);
   return cudaLaunchKernelEx(&cfg, fn, a);
 }
 
 template <typename TW>
-cudaError_t launch_pipe_np(cudaStream_t st, PipeArgs& a, int B, int np, size_t smem) {
+cudaError_t pipe_np(cudaStream_t st, const PipeArgs& a, int B, int np, size_t smem, int* active) {
   switch (np) {
-    case 2: return launch_pipe<TW, 2>(st, a, B, smem);
-    case 4: return launch_pipe<TW, 4>(st, a, B, smem);
-    case 5: return launch_pipe<TW, 5>(st, a, B, smem);
-    case 6: return launch_pipe<TW, 6>(st, a, B, smem);
-    default: return launch_pipe<TW, 8>(st, a, B, smem);
+    case 2: return pipe_launch<TW, 2>(st, a, B, smem, active);
+    case 4: return pipe_launch<TW, 4>(st, a, B, smem, active);
+    case 5: return pipe_launch<TW, 5>(st, a, B, smem, active);
+    case 6: return pipe_launch<TW, 6>(st, a, B, smem, active);
+    default: return pipe_launch<TW, 8>(st, a, B, smem, active);
   }
+}
+
+template <typename TW>
+int pipe_active(const PipeArgs& a, int np, size_t smem) {
+  int n = 0;
+  if (pipe_np<TW>(nullptr, a, 1, np, smem, &n) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 }  // namespace
@@ -675,7 +754,7 @@ cudaError_t launch_pipe_np(cudaStream_t st, PipeArgs& a, int B, int np, size_t s
 cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,
                               int B, int d, int steps, const float* theta, const void* wbf,
                               const int64_t (*off_w)[3], int64_t off_wy, int64_t off_by,
-                              const float* window, float* out, int sms) {
+                              const float* window, float* out, unsigned* status) {
   if (L > 4 || T > 16) return cudaErrorInvalidConfiguration;
   const int np = T <= 4 ? 2 : (T <= 8 ? 4 : (T <= 10 ? 5 : (T <= 12 ? 6 : 8)));
   const size_t wsz = bf16_weights ? 2 : 4;
@@ -689,33 +768,38 @@ cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, 
   a.off_by = off_by;
   a.window = window;
   a.out = out;
-  // the largest cluster that leaves a CTA four units and lets the samples'
-  // clusters run in at most two waves; if none does, the smallest whose CTAs
-  // hold their weights
-  int pick = 0;
+  a.status = status;
+  // Cluster size: the waves that the B clusters need at that size times one
+  // row's time, its products at the FP32 rate plus a fixed latency per layer
+  // (partial sums, gates, exchange: about 1500 clocks).  Sizes above 8 are
+  // the non-portable ones; at 2 x 256 seven clusters of 16 run at once, or
+  // eight of 12, so 8 samples take 12 (one wave).
   auto shape = [&](int CS) {
     a.CS = CS;
-    a.U = (H + CS - 1) / CS;
-    const int R = 4 * a.U;
-    a.LR = 1;
-    while (a.LR < 32 && 2 * a.LR < R) a.LR <<= 1;
-    a.SUB = 32 / a.LR;
-    a.RB = 1;
-    while (64 * a.RB < R) a.RB <<= 1;
-    if (a.RB > kPipeWarps) return (size_t)-1;
-    a.SL = kPipeWarps / a.RB * a.SUB;
-    return pipe_smem_bytes(I, H, L, O, a.U, CS, 2 * np, a.SL, wsz);
+    a.U = even_up((H + CS - 1) / CS);
+    a.SL = std::min(kPipeThreads / (2 * a.U), std::max(1, std::min(16, H / 8)));
+    a.threads = a.SL * 2 * a.U;
+    return a.SL < 1 ? (size_t)-1 : pipe_smem_bytes(I, H, L, O, a.U, CS, 2 * np, a.SL, wsz);
   };
-  for (int CS = 16; CS >= 1; CS >>= 1) {
-    if (CS > 1 && (H + CS - 1) / CS < 4) continue;
-    if (shape(CS) > (size_t)227 * 1024) break;
-    pick = CS;
-    if ((int64_t)B * CS <= 2 * sms) break;
+  int pick = 0;
+  double best = 0.0;
+  for (int CS : {16, 12, 8, 4, 2, 1}) {
+    const size_t smem = shape(CS);
+    if (smem > (size_t)226 * 1024 || (CS > 1 && H < 2 * CS)) continue;
+    const int active = bf16_weights ? pipe_active<__nv_bfloat16>(a, np, smem)
+                                    : pipe_active<float>(a, np, smem);
+    if (active < 1) continue;
+    const double products = 4.0 * a.U * 2 * np * (2.0 * L - 1.0) * H / 128.0;
+    const double cost = (double)((B + active - 1) / active) * (1.5 * products + 1500.0 * L);
+    if (!pick || cost < best) {
+      pick = CS;
+      best = cost;
+    }
   }
   if (!pick) return cudaErrorInvalidConfiguration;
   const size_t smem = shape(pick);
-  const cudaError_t e = bf16_weights ? launch_pipe_np<__nv_bfloat16>(st, a, B, np, smem)
-                                     : launch_pipe_np<float>(st, a, B, np, smem);
+  const cudaError_t e = bf16_weights ? pipe_np<__nv_bfloat16>(st, a, B, np, smem, nullptr)
+                                     : pipe_np<float>(st, a, B, np, smem, nullptr);
   if (e == cudaSuccess) note_launch();
   return e;
 }
