@@ -538,9 +538,13 @@ k_eig_cluster(int l, const float* __restrict__ sd, const float* __restrict__ se,
     Xs[r * ldx + g] = Z[e];
   }
   __syncthreads();
-  // orthogonalise vectors of close eigenvalues.  Per vector a of a
+  // orthogonalise vectors of close eigenvalues, the largest of a cluster
+  // first: the gap test is absolute, so the small end of a graded spectrum
+  // is one cluster, and its larger eigenvalues' vectors are accurate where
+  // the smallest ones', below the rounding of T, are noise that must not be
+  // subtracted from them.  Per vector a of a
   // cluster, two classical Gram-Schmidt passes against the cluster's
-  // earlier (already orthonormal) vectors: the dots by one warp each, the
+  // vectors above a (already orthonormal): the dots by one warp each, the
   // update by 16 threads per row.  A vector that loses more than half its
   // norm (a multiple eigenvalue) is replaced by warp 0: inverse iteration
   // with T - lambda I from a pseudo-random vector, which keeps the
@@ -563,9 +567,9 @@ k_eig_cluster(int l, const float* __restrict__ sd, const float* __restrict__ se,
     int start = 0, nrep = 0;
     for (int i = 1; i <= l; ++i) {
       if (i < l && lam[i] - lam[i - 1] <= ctol) continue;
-      for (int a = start + 1; a < i; ++a) {
+      for (int a = i - 2; a >= start; --a) {
         for (int pass = 0; pass < 2; ++pass) {
-          for (int b = start + warp; b < a; b += nt >> 5) {
+          for (int b = a + 1 + warp; b < i; b += nt >> 5) {
             float dt = 0.f;
             for (int r = lane; r < l; r += 32) dt = fmaf(Xs[r * ldx + b], Xs[r * ldx + a], dt);
             dt = warp_sum(dt);
@@ -576,7 +580,7 @@ k_eig_cluster(int l, const float* __restrict__ sd, const float* __restrict__ se,
             const int r = r0 + rsub;
             float acc = 0.f;
             if (r < l)
-              for (int b = start + part; b < a; b += 16) acc = fmaf(dts[b], Xs[r * ldx + b], acc);
+              for (int b = a + 1 + part; b < i; b += 16) acc = fmaf(dts[b], Xs[r * ldx + b], acc);
             acc += __shfl_xor_sync(hmask, acc, 1);
             acc += __shfl_xor_sync(hmask, acc, 2);
             acc += __shfl_xor_sync(hmask, acc, 4);
@@ -668,7 +672,7 @@ k_eig_cluster(int l, const float* __restrict__ sd, const float* __restrict__ se,
               xa[u] = r < l ? s_iv[r] : 0.f;
             }
             for (int rep = 0; rep < 2; ++rep)
-              for (int b = start; b < a; ++b) {
+              for (int b = a + 1; b < i; ++b) {
                 float xb[4], dt = 0.f;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
