@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "rpod_internal.cuh"
+#include "rpod_split.cuh"
 #include "rpod_tc.cuh"
 
 using namespace rpod;
@@ -57,6 +58,8 @@ struct rpod_plan {
   // side stream and fork/join events (16-bit forms: the last CholeskyQR
   // round runs beside the refinement pass); null when they could not be made
   cudaStream_t side;
+  size_t off_planes;  // FP32 form: the parts of a product's skinny operand
+  int split_pct;      // share of the default split-K of the split FP32 products
   cudaEvent_t ev_fork, ev_join;
   // graph replay of repeated basis calls: the second call with the same
   // buffers captures the launch sequence (on gcap) into gexec, later calls
@@ -127,6 +130,16 @@ int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
     if (r_ != RPOD_OK) return r_;                    \
   } while (0)
 
+// FP32 form, FP64 factorization of an ill-conditioned first round: the Gram's
+// diagonal is raised by this share, (1e-6)^2, as rounding noise of 1e-6 in
+// every column of the sampled matrix would raise it.  FP32 FMA sums over S left
+// about that much; the split products leave 1e-7, and a factor X = R^{-1} that
+// resolves columns so far down (entries near 1e7, in FP32) puts errors of order
+// one into Q = Y X and loses columns in the next round: for nine of twelve
+// sketches of a spectrum that falls to 1e-7 sigma_1 within l = 80, and for none
+// with the raised diagonal (sigma down to 1e-4 sigma_1 within 2e-6 in all).
+constexpr double kF32Reg = 1e-12;
+
 // ---------------------------------------------------------------------------
 // Pipelines on working type W (double for RPOD_F64, float otherwise).
 template <typename W>
@@ -145,6 +158,26 @@ struct Run {
   int exchange(void* p, int64_t count, int dtype, int op) {
     if (!P->rows_mode) return RPOD_OK;
     return P->xch(P->xch_ctx, p, count, dtype, op, (void*)st) == 0 ? RPOD_OK : RPOD_ERR_EXCHANGE;
+  }
+
+  // D(i, c) (at D[i di + c dj]) = sum_k A(i, k) B(k, c), c < N: FP64 on the
+  // SIMT pipes (split into nsplit ranges of k summed from off_part, di == 1),
+  // FP32 on the tensor cores with exactly split operands (rpod_split.cu)
+  int product(bool kc, int64_t M, int N, int64_t K, int nsplit, const W* A, int64_t lda, const W* B,
+              int64_t ldb, W* D, int64_t di, int64_t dj, bool check) {
+    if constexpr (sizeof(W) == 4) {
+      return split_gemm(st, kc, M, N, K, A, lda, B, ldb, D, di, dj, ws + P->off_planes,
+                        (float*)(ws + P->off_part), P->part_elems, P->split_pct, status, check);
+    } else {
+      if (nsplit <= 1) {
+        CK((gemm<W, W, W, W>(st, kc, M, N, K, 1, A, lda, B, ldb, D, di, dj, 0, status, check)));
+      } else {
+        W* part = buf(P->off_part);
+        CK((gemm<W, W, W, W>(st, kc, M, N, K, nsplit, A, lda, B, ldb, part, 1, M, M * N, status, check)));
+        CK((reduce_splits<W, W>(st, M, N, nsplit, part, D, di, dj)));
+      }
+      return RPOD_OK;
+    }
   }
 
   // Gram G = A^T A (A rows x l, ld lda) in FP64: products in W, summed in W
@@ -221,7 +254,8 @@ struct Run {
     // direction; the callers add one round for it
     const double grows = (dist && P->rows_mode) ? (double)P->n_total : (double)rows;
     const double shift_coef =
-        sizeof(W) == 8 ? 11.0 * (grows * l + (double)l * (l + 1)) * (DBL_EPSILON / 2) : 0.0;
+        sizeof(W) == 8 ? 11.0 * (grows * l + (double)l * (l + 1)) * (DBL_EPSILON / 2)
+                       : (P->compute == RPOD_F32 ? kF32Reg : 0.0);
     for (int r = 0; r < rounds; ++r) {
       double* G = dbuf(P->off_g);
       CR(gram(src, rows, ld, G, ns, !(exact_last && r == rounds - 1)));
@@ -243,9 +277,13 @@ struct Run {
                       status);
       if (rc == RPOD_ERR_CUDA) return rc;
       if (tco && last_apply) tco->used = rc == RPOD_OK;
-      if (rc != RPOD_OK)
-        CK((gemm<W, W, W, W>(st, false, rows, l, l, 1, src, ld, buf(P->off_xw), l, dst, 1, ld, 0,
-                             status, false)));
+      if (rc != RPOD_OK) {
+        if (P->compute == RPOD_F32)
+          CR(product(false, rows, l, l, 1, src, ld, buf(P->off_xw), l, dst, 1, ld, false));
+        else
+          CK((gemm<W, W, W, W>(st, false, rows, l, l, 1, src, ld, buf(P->off_xw), l, dst, 1, ld, 0,
+                               status, false)));
+      }
       W* t = src; src = dst; dst = t;
     }
     *out = src;
@@ -279,9 +317,13 @@ struct Run {
       rc = tc_apply(st, (const float*)Tt1, m, m, l, (const float*)buf(P->off_xw), l, (float*)out, m,
                     0, nullptr, 0, nullptr, 0, status, 0, true);
     if (rc == RPOD_ERR_CUDA) return rc;
-    if (rc != RPOD_OK)
-      CK((gemm<W, W, W, W>(st, false, m, l, l, 1, Tt1, m, buf(P->off_xw), l, out, 1, m, 0, status,
-                           false)));
+    if (rc != RPOD_OK) {
+      if (P->compute == RPOD_F32)
+        CR(product(false, m, l, l, 1, Tt1, m, buf(P->off_xw), l, out, 1, m, false));
+      else
+        CK((gemm<W, W, W, W>(st, false, m, l, l, 1, Tt1, m, buf(P->off_xw), l, out, 1, m, 0, status,
+                             false)));
+    }
     return RPOD_OK;
   }
 
@@ -340,8 +382,12 @@ struct Run {
       rc = tc_apply(st, (const float*)Q, n, n, l, (const float*)Uw, l, (float*)U, ldu, 0, nullptr, 0,
                     nullptr, 0, status, ku, true);
     if (rc == RPOD_ERR_CUDA) return rc;
-    if (rc != RPOD_OK)
-      CK((gemm<W, W, W, W>(st, false, n, ku, l, 1, Q, n, Uw, l, U, 1, ldu, 0, status, false)));
+    if (rc != RPOD_OK) {
+      if (P->compute == RPOD_F32)
+        CR(product(false, n, ku, l, 1, Q, n, Uw, l, U, 1, ldu, false));
+      else
+        CK((gemm<W, W, W, W>(st, false, n, ku, l, 1, Q, n, Uw, l, U, 1, ldu, 0, status, false)));
+    }
     if (P->rows_mode) {
       // the largest-magnitude entry of each column over all row blocks (ties
       // to the lowest global row) decides its sign: three exchanges of l
@@ -360,6 +406,8 @@ struct Run {
     }
     // Sec. 4.3 coefficients C = U_k^T S = Uhat_k^T T (k x m), Uhat with the signs
     CK((convert_matrix<double, W>(st, l, k, Uhat, l, Uw, l)));
+    if (P->compute == RPOD_F32)
+      return product(false, m, k, l, 1, Tt, m, Uw, l, C, ldc, 1, false);
     CK((gemm<W, W, W, W>(st, false, m, k, l, 1, Tt, m, Uw, l, C, ldc, 1, 0, status, false)));
     return RPOD_OK;
   }
@@ -373,7 +421,6 @@ struct Run {
     W* Z = buf(P->off_z);
     W* Zq = buf(P->off_zq);
     W* Tt = buf(P->off_tt);
-    W* part = buf(P->off_part);
     const double sw = sizeof(W);
     const double pass_bytes = sw * ((double)n * m + (double)n * l + (double)m * l);
     const double pass_flops = 2.0 * n * m * l;
@@ -383,22 +430,20 @@ struct Run {
     CK((sketch<W>(st, P->seed, 0, m, l, Lam, m)));
     // Alg. 1: P = S Lambda (pass over S; flags non-finite input)
     prof_begin(P, st);
-    CK((gemm<W, W, W, W>(st, false, n, l, m, 1, S, lds, Lam, m, Y, 1, n, 0, status, true)));
+    CR(product(false, n, l, m, 1, S, lds, Lam, m, Y, 1, n, true));
     prof_end(P, st, pass_bytes, pass_flops);
     W* Q = nullptr;
     for (int it = 0; it <= q; ++it) {
       if (it > 0) {
         // Alg. 1 subspace iteration: Z = S^T Q, orthonormalise, Y = S Z
         prof_begin(P, st);
-        CK((gemm<W, W, W, W>(st, true, m, l, n, P->nsplit_z, S, lds, Q, n, part, 1, m, m * l,
-                             status, false)));
+        CR(product(true, m, l, n, P->nsplit_z, S, lds, Q, n, Z, 1, m, false));
         prof_end(P, st, pass_bytes, pass_flops);
-        CK((reduce_splits<W, W>(st, m, l, P->nsplit_z, part, Z, 1, m)));
         CR(exchange(Z, m * l, sizeof(W) == 8 ? RPOD_F64 : RPOD_F32, RPOD_REDUCE_SUM));
         W* Zo = nullptr;
         CR(orth(Z, Zq, m, 1 + extra, &Zo, false));
         prof_begin(P, st);
-        CK((gemm<W, W, W, W>(st, false, n, l, m, 1, S, lds, Zo, m, Y, 1, n, 0, status, false)));
+        CR(product(false, n, l, m, 1, S, lds, Zo, m, Y, 1, n, false));
         prof_end(P, st, pass_bytes, pass_flops);
       }
       // Alg. 1 QR of the sampled matrix (CholeskyQR2 for the final basis);
@@ -408,10 +453,8 @@ struct Run {
     // Alg. 1: T = Q^T S, stored transposed (m x l), with the deferred last
     // CholeskyQR factor folded in afterwards
     prof_begin(P, st);
-    CK((gemm<W, W, W, W>(st, true, m, l, n, P->nsplit_z, S, lds, Q, n, part, 1, m, m * l, status,
-                         false)));
+    CR(product(true, m, l, n, P->nsplit_z, S, lds, Q, n, Zq, 1, m, false));
     prof_end(P, st, pass_bytes, pass_flops);
-    CK((reduce_splits<W, W>(st, m, l, P->nsplit_z, part, Zq, 1, m)));
     CR(exchange(Zq, m * l, sizeof(W) == 8 ? RPOD_F64 : RPOD_F32, RPOD_REDUCE_SUM));
     CR(fold_t(Zq, Tt));
     return finish(Q, Tt, U, ldu, sigma, C, ldc, true);
@@ -545,12 +588,13 @@ struct Run {
     const bool refine = refine_req;
     const bool ref_tma = refine_tma;
     if (refine && !ref_tma) {
-      // FP32 copy not addressable by TMA: the SIMT FP32 pass computes T
+      // FP16 form, or an FP32 copy not addressable by TMA: products as
+      // accurate as FP32 ones (the 16-bit operands and the TF32 basis are
+      // free by now and hold Q's parts)
       prof_begin(P, st);
-      CK((gemm<float, float, float, float>(st, true, m, l, n, P->nsplit_z, Sref, ldr, Q, n,
-                                           (float*)buf(P->off_part), 1, m, m * l, status, false)));
+      CR(split_gemm(st, true, m, l, n, Sref, ldr, Q, n, Zq, 1, m, ws + P->off_qb,
+                    (float*)(ws + P->off_part), P->part_elems, P->split_pct, status, false));
       prof_end(P, st, 4.0 * ((double)n * m + (double)n * l + (double)m * l), pass_flops);
-      CK((reduce_splits<float, float>(st, m, l, P->nsplit_z, (float*)buf(P->off_part), Zq, 1, m)));
       CK(join());
       CR(fold_t(Zq, Tt));
       return finish(Q, Tt, U, ldu, sigma, C, ldc, true);
@@ -575,18 +619,27 @@ struct Run {
   int project(const W* U, int64_t ldu, int kc, const W* Sn, int64_t lds, int64_t mn, W* C,
               int64_t ldc) {
     const int64_t n = P->n;
-    // C'^T (mn x kc) = S'^T U, split over n, chunked over snapshots so the
-    // partial buffer of the plan suffices
-    const int64_t per = (int64_t)(P->part_elems / ((size_t)P->nsplit_z * (size_t)kc));
-    const int64_t cols = per < 1 ? 1 : per;
-    for (int64_t j0 = 0; j0 < mn; j0 += cols) {
-      const int64_t mc = (mn - j0 < cols) ? (mn - j0) : cols;
-      W* part = buf(P->off_part);
-      CK((gemm<W, W, W, W>(st, true, mc, kc, n, P->nsplit_z, Sn + j0 * lds, lds, U, ldu, part, 1, mc,
-                           mc * kc, status, false)));
-      CK((reduce_splits<W, W>(st, mc, kc, P->nsplit_z, part, C + j0 * ldc, ldc, 1)));
+    if constexpr (sizeof(W) == 4) {
+      // U's parts go where the plan's passes keep their 16-bit operands
+      const bool h = is16(P->compute) && P->wpart_elems > P->part_elems;
+      return split_gemm(st, true, mn, kc, n, Sn, lds, U, ldu, C, ldc, 1,
+                        ws + (is16(P->compute) ? P->off_qb : P->off_planes),
+                        (float*)(ws + (h ? P->off_wpart : P->off_part)),
+                        h ? P->wpart_elems : P->part_elems, 100, status, false);
+    } else {
+      // C'^T (mn x kc) = S'^T U, split over n, chunked over snapshots so the
+      // partial buffer of the plan suffices
+      const int64_t per = (int64_t)(P->part_elems / ((size_t)P->nsplit_z * (size_t)kc));
+      const int64_t cols = per < 1 ? 1 : per;
+      for (int64_t j0 = 0; j0 < mn; j0 += cols) {
+        const int64_t mc = (mn - j0 < cols) ? (mn - j0) : cols;
+        W* part = buf(P->off_part);
+        CK((gemm<W, W, W, W>(st, true, mc, kc, n, P->nsplit_z, Sn + j0 * lds, lds, U, ldu, part, 1,
+                             mc, mc * kc, status, false)));
+        CK((reduce_splits<W, W>(st, mc, kc, P->nsplit_z, part, C + j0 * ldc, ldc, 1)));
+      }
+      return RPOD_OK;
     }
-    return RPOD_OK;
   }
 
   // 16-bit S': the W-pass with U converted to the 16-bit operand layout.
@@ -666,6 +719,15 @@ static int plan_create_impl(rpod_plan** out, int64_t n, int64_t m, int32_t k, in
   P->split_cap = split_cap < 1 ? 1 : split_cap;
   P->nsz_def = P->nsplit_z;
   P->part_elems = std::max((size_t)P->nsplit_z * P->split_cap * m * L, (size_t)1);
+  P->split_pct = 100;
+  if (compute != RPOD_F64) {
+    // partial sums of the split FP32 products: the passes of the FP32 form,
+    // the FP16 form's refinement pass and projections
+    const size_t cap = std::max(P->part_elems, (size_t)32 << 20);
+    P->part_elems = std::max(P->part_elems, (size_t)split_count(m, n, (int)l, cap) * m * L);
+    const int sy = compute == RPOD_F32 ? split_count(n, m, (int)l, cap) : 1;
+    if (sy > 1) P->part_elems = std::max(P->part_elems, (size_t)sy * n * L);
+  }
   P->gpart_elems = std::max((size_t)nsg, (size_t)P->nsplit_t) * L * L;
   P->sign_bytes = sign_fix_scratch_bytes(n, (int)L);
   size_t off = 0;
@@ -690,6 +752,8 @@ static int plan_create_impl(rpod_plan** out, int64_t n, int64_t m, int32_t k, in
   P->off_xch = take(8 * 6 * L);
   P->n_ld = round_up(n, 64);
   P->m_ld = round_up(m, 64);
+  P->off_planes = 0;
+  if (compute == RPOD_F32) P->off_planes = take(split_plane_bytes(std::max(n, m), (int)l));
   P->off_sb = P->off_qb = P->off_zb = P->off_atf = P->off_wpart = 0;
   P->nsplit_w = 0;
   P->wpart_elems = 0;
@@ -1125,6 +1189,7 @@ void apply_split(rpod_plan* P, int pct) {
     return s;
   };
   P->nsplit_z = scale(P->nsz_def);
+  P->split_pct = pct;
   if (P->nsw_def > 0) P->nsplit_w = scale(P->nsw_def);
 }
 

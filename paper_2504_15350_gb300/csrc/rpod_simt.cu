@@ -1022,7 +1022,7 @@ template <typename TW>
 __global__ void __launch_bounds__(256)
 k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
                    double* __restrict__ Xout, TW* __restrict__ Xw, int ldxw, unsigned* status,
-                   double* __restrict__ part, int nsplit, unsigned* ticket);
+                   double* __restrict__ part, int nsplit, unsigned* ticket, double reg);
 
 // Gram partials of an FP32 matrix with exact products, run only when the
 // gate is raised (an FP32 Gram cannot resolve pivots below about 1e-9 of the
@@ -1153,7 +1153,7 @@ cudaError_t cholesky(cudaStream_t st, int l, const void* Gv, double tol, int rou
   const size_t sm64 = gated_smem_bytes(l);
   const unsigned grid = gp && nsplit > 1 ? (unsigned)(((int64_t)l * l + 63) / 64) : 1u;
   k_cholesky64_gated<TW><<<grid, 256, sm64, st>>>(l, nullptr, 1e-13, gate, X, Xw, ldxw, status, gp,
-                                                  nsplit, status + 9);
+                                                  nsplit, status + 9, shift_coef);
   note_launch();
   return cudaGetLastError();
 }
@@ -1162,7 +1162,7 @@ template <typename TW>
 __global__ void __launch_bounds__(256)
 k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
                    double* __restrict__ Xout, TW* __restrict__ Xw, int ldxw, unsigned* status,
-                   double* __restrict__ part, int nsplit, unsigned* ticket) {
+                   double* __restrict__ part, int nsplit, unsigned* ticket, double reg) {
   __shared__ int s_go, s_last;
   __shared__ double s_zs[8][32];
   if (threadIdx.x == 0) s_go = *gate;
@@ -1220,7 +1220,7 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
     if (i > j) continue;
     // split 0 holds the sums (written by other CTAs: read through L2)
     const double g = part ? (nsplit > 1 ? __ldcg(part + e) : part[e]) : G[e];
-    A[i + j * ld] = g;
+    A[i + j * ld] = i == j ? g + reg * g : g;
     if (i == j) d0[j] = g;
   }
   __syncthreads();
