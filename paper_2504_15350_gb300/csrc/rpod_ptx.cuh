@@ -67,9 +67,10 @@ __device__ __forceinline__ uint64_t gtimer() {
   return t;
 }
 // Bounded wait on a phase; false when the deadline passed or another role
-// already gave up (the shared abort flag).
-static __device__ __noinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try(b, parity)) return true;
+// already gave up (the shared abort flag).  The first try is inlined: the
+// call alone, usually on a phase that is already complete, cost the MMA
+// issuer about 100 clocks per wait.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
   const uint64_t t0 = gtimer();
   while (true) {
     if (mbar_try(b, parity)) return true;
@@ -79,6 +80,9 @@ static __device__ __noinline__ bool mbar_wait(uint64_t* b, uint32_t parity, vola
       return false;
     }
   }
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  return mbar_try(b, parity) || mbar_wait_slow(b, parity, abort_flag);
 }
 // Bounded wait that ignores the abort flag: used after an abort to let this
 // thread's own copies or MMAs finish before the shared memory and TMEM they
@@ -111,6 +115,16 @@ __device__ __forceinline__ void tc_before() {
 }
 __device__ __forceinline__ void tc_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// One lane of a converged warp.  The roles of a single thread (TMA, MMA) are
+// entered through it rather than through lane == 0: the compiler then knows
+// that one thread runs and keeps descriptors and addresses in uniform
+// registers, without which an MMA took about 65 clocks to issue whatever its
+// shape.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+  return p != 0;
 }
 template <int KIND>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {

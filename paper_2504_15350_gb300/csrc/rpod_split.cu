@@ -51,8 +51,8 @@ namespace tc {
 
 template <int NT>
 struct SplitSmem {
-  static constexpr int RS = NT == 128 ? 3 : 4;                 // raw slots
-  static constexpr int BS = NT >= 96 ? 2 : (NT == 64 ? 3 : 4); // B stages
+  static constexpr int RS = NT == 128 ? 2 : (NT == 96 ? 3 : 4);  // raw slots
+  static constexpr int BS = NT == 32 ? 4 : 3;                    // B stages
   static constexpr uint32_t RAW = 32768;
   static constexpr uint32_t PLANE = NT * 128;
   static constexpr uint32_t BST = 3 * PLANE;
@@ -158,7 +158,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 
   // Every role walks over the same items and counts k-blocks in `it`.
   if (warp == 0 && TMA) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool go = true;
       for (int64_t w = blockIdx.x; w < g.items && go; w += gridDim.x) {
@@ -183,7 +183,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           mbar_wait_drain(&rfull[j % RS], (uint32_t)(j / RS) & 1u);
     }
   } else if (warp == 18) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool go = true;
       for (int64_t w = blockIdx.x; w < g.items && go; w += gridDim.x) {
@@ -203,7 +203,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           mbar_wait_drain(&bfull[j % BS], (uint32_t)(j / BS) & 1u);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t id = idesc(1, false, 128, NT);
       int it = 0;
       bool go = true;

@@ -84,7 +84,7 @@ k_wpass(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0 && nk > 0) {
+  if (warp == 0 && nk > 0 && elect_one()) {
     for (int it = 0; it < nk; ++it) {
       const int s = it % STAGES;
       const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
@@ -118,7 +118,7 @@ k_wpass(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       __syncwarp();
       if (lane == 0) mbar_arrive(&conv[s]);
     }
-  } else if (warp == 1 && lane == 0 && nk > 0) {
+  } else if (warp == 1 && nk > 0 && elect_one()) {
     constexpr uint32_t id = idesc(fmt_of(KIND), false, 128, BN);
     int it = 0;
     for (; it < nk; ++it) {
@@ -214,7 +214,7 @@ k_ypass(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     for (int j = 0; j < nk; ++j) {
       const int s = j % STAGES;
       const uint32_t ph = (uint32_t)(j / STAGES) & 1u;
@@ -227,7 +227,7 @@ k_ypass(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtenso
       for (int b = 0; b < BN / 64; ++b)
         tma_load_2d(a + L::A_BYTES + b * 8192, &tmS, &full[s], (int)(i0 + 64 * b), it * 64);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     constexpr uint32_t id = idesc(fmt_of(KIND), true, 128, BN);
     for (int j = 0; j < nk; ++j) {
       const int s = j % STAGES;
@@ -327,7 +327,7 @@ k_gram3(const __grid_constant__ CUtensorMap tmY, int64_t rows, int l, int kchunk
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0 && nk > 0) {
+  if (warp == 0 && nk > 0 && elect_one()) {
     for (int it = 0; it < nk; ++it) {
       const int s = it % STAGES;
       const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
@@ -358,7 +358,7 @@ k_gram3(const __grid_constant__ CUtensorMap tmY, int64_t rows, int l, int kchunk
       __syncwarp();
       if (lane == 0) mbar_arrive(&conv[s]);
     }
-  } else if (warp == 1 && lane == 0 && nk > 0) {
+  } else if (warp == 1 && nk > 0 && elect_one()) {
     constexpr uint32_t id = idesc(2, false, 128, 128);
     for (int it = 0; it < nk; ++it) {
       const int s = it % STAGES;
@@ -475,7 +475,7 @@ k_gram_x(const __grid_constant__ CUtensorMap tmY, int64_t rows, int l, int kchun
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     int it = 0;
     for (; it < nk; ++it) {
       const int s = it % STAGES;
@@ -512,7 +512,7 @@ k_gram_x(const __grid_constant__ CUtensorMap tmY, int64_t rows, int l, int kchun
       __syncwarp();
       if (lane == 0) mbar_arrive(&conv[s]);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     constexpr uint32_t id = idesc(2, false, 128, 128);
     bool go = true, issued = false;
     for (int ch = 0, it = 0; ch < nch && go; ++ch) {
@@ -654,7 +654,7 @@ k_ypass_cvt(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     for (int j = 0; j < nk; ++j) {
       const int s = j % STAGES;
       const uint32_t ph = (uint32_t)(j / STAGES) & 1u;
@@ -713,7 +713,7 @@ k_ypass_cvt(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       if (lane == 0) mbar_arrive(&conv[s]);
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, ST_NONFINITE);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     constexpr uint32_t id = idesc(fmt_of(KIND), true, 128, BN);
     for (int j = 0; j < nk; ++j) {
       const int s = j % STAGES;
@@ -889,7 +889,7 @@ k_apply_tf32(const __grid_constant__ CUtensorMap tmY, const float* __restrict__ 
   tc_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     int it = 0;  // loads issued
     bool go = true;
     for (int lt = 0; lt < nlt && go; ++lt) {
@@ -968,7 +968,7 @@ k_apply_tf32(const __grid_constant__ CUtensorMap tmY, const float* __restrict__ 
           mbar_arrive(&cfull[c]);
         }
       }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     constexpr uint32_t id = idesc(2, false, 128, 128);
     bool go = true, issued = false;
     for (int lt = 0, it = 0; lt < nlt && go; ++lt) {
