@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "rpod_internal.cuh"
+#include "rpod_lstm_mma.cuh"
 
 struct rpod_lstm {
   int I, H, L, O, T, Bmax;
@@ -47,6 +48,8 @@ struct rpod_lstm {
   double drop_p;
   uint64_t drop_seed, drop_thr;
   int64_t drop_pass;
+  size_t o_keep;   // dropout masks of layers 1..L-1 (bytes, as o_xd)
+  size_t o_lpart;  // the head's shares of the loss
   size_t o_xd;  // masked inputs of layers 1..L-1 (T x Bmax x H each)
   size_t o_bx, o_by, o_lsum;  // train_epoch: the gathered batch, the loss sum
   size_t o_sync;  // persistent rollout: barrier arrivals, abort word, status word
@@ -97,13 +100,9 @@ __global__ void k_to_time_major(int B, int T, int I, const float* __restrict__ X
 // One recurrent step of one layer for all batch rows: 256 threads, tile of
 // 32 batch rows x 32 units (x 4 gates); thread (tb, tu) holds 4 rows x 4 gates
 // of unit u0 + tu.
-__device__ __forceinline__ float ldw(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-__device__ __forceinline__ float ldw(const float* p) { return *p; }
-
-template <typename TW>
 __global__ void __launch_bounds__(256)
 k_lstm_fwd_step(int B, int H, const float* __restrict__ Gx, const float* __restrict__ bias,
-                const float* __restrict__ h_prev, const TW* __restrict__ Wh,
+                const float* __restrict__ h_prev, const float* __restrict__ Wh,
                 const float* __restrict__ c_prev, float* __restrict__ c_out, float* __restrict__ h_out,
                 float* __restrict__ gates) {
   __shared__ float hs[32][33];
@@ -125,7 +124,7 @@ k_lstm_fwd_step(int B, int H, const float* __restrict__ Gx, const float* __restr
       const int rr = e >> 5, kk = e & 31;
       const int g = rr >> 5, uu = rr & 31;
       const int u = u0 + uu, k = k0 + kk;
-      wsm[rr][kk] = (u < H && k < H) ? ldw(Wh + (int64_t)(g * H + u) * H + k) : 0.f;
+      wsm[rr][kk] = (u < H && k < H) ? Wh[(int64_t)(g * H + u) * H + k] : 0.f;
     }
     __syncthreads();
 #pragma unroll 8
@@ -338,29 +337,140 @@ struct Net {
     return RPOD_OK;
   }
 
-  template <typename TW>
-  const TW* weights() const {
-    return sizeof(TW) == 4 ? (const TW*)(ws + N->o_theta) : (const TW*)(ws + N->o_wbf);
+  // y (B x O) of the time-major input Xt (T x B x I); with a target also dy and
+  // (FP32 weights) the loss.  BF16 weights: tensor-core cells, one launch per
+  // anti-diagonal (rpod_lstm_mma.cu); FP32 weights: the SIMT kernels here.
+  int forward(const float* Xt, int B, float* y, const float* tgt) {
+    if (!N->wfp32) return forward_mma(Xt, B, y, tgt);
+    CR2(forward_simt(Xt, B, y));
+    k_head_loss<<<1, 1024, 0, st>>>(B, N->O, y, f(N->o_theta) + N->off_by, tgt, f(N->o_dy), f(N->o_loss));
+    LL();
+    return RPOD_OK;
   }
-  int forward(const float* Xt, int B) {
-    return N->wfp32 ? forward_t<float>(Xt, B) : forward_t<__nv_bfloat16>(Xt, B);
-  }
+  // every gradient into o_grad (BF16 weights: and the loss into o_loss)
   int backward(const float* Xt, int B) {
-    return N->wfp32 ? backward_t<float>(Xt, B) : backward_t<__nv_bfloat16>(Xt, B);
+    return N->wfp32 ? backward_simt(Xt, B) : backward_mma(Xt, B);
+  }
+
+  float drop_scale() const { return (float)(1.0 / (1.0 - N->drop_p)); }
+  unsigned char* keep(int l) const {  // mask of the input of layer l >= 1
+    return (unsigned char*)(ws + N->o_keep) + (size_t)(l - 1) * N->T * N->Bmax * N->H;
+  }
+
+  int forward_mma(const float* Xt, int B, float* y, const float* tgt) {
+    const int H = N->H, T = N->T, L = N->L;
+    const int64_t BH = (int64_t)B * H;
+    LstmFwd a;
+    a.B = B;
+    a.H = H;
+    a.drop_seed = N->drop_seed;
+    a.drop_pass = (uint64_t)N->drop_pass;
+    a.drop_thr = N->drop_thr;
+    a.drop_scale = drop_scale();
+    for (int ph = 0; ph < L + T - 1; ++ph) {
+      a.cells = 0;
+      for (int l = 0; l < L; ++l) {
+        const int t = ph - l;
+        if (t < 0 || t >= T) continue;
+        LstmFwdCell& c = a.cell[a.cells++];
+        c.Il = in_dim(l);
+        c.x = l == 0 ? Xt + (size_t)t * B * N->I : layer_input(l, B) + t * BH;
+        c.hprev = t > 0 ? hh(l) + t * BH : nullptr;
+        c.cprev = t > 0 ? cc(l) + t * BH : nullptr;
+        c.Wx = wbf() + N->off_w[l][0];
+        c.Wh = wbf() + N->off_w[l][1];
+        c.bias = f(N->o_theta) + N->off_w[l][2];
+        c.c = cc(l) + (t + 1) * BH;
+        c.h = hh(l) + (t + 1) * BH;
+        c.gates = gates(l) + t * 4 * BH;
+        const bool drop = train_drop && l + 1 < L;
+        c.xd = drop ? xd(l + 1) + t * BH : nullptr;
+        c.keep = drop ? keep(l + 1) + t * BH : nullptr;
+        c.drop_layer = (uint64_t)(l + 1);
+        c.drop_e0 = t * BH;
+      }
+      LK(lstm_fwd_phase(st, a));
+    }
+    LK(lstm_head(st, B, N->O, H, hh(L - 1) + T * BH, wbf() + N->off_wy, f(N->o_theta) + N->off_by, y, tgt,
+                 f(N->o_dy), (double*)(ws + N->o_lpart)));
+    return RPOD_OK;
+  }
+
+  int backward_mma(const float* Xt, int B) {
+    const int H = N->H, T = N->T, L = N->L, O = N->O;
+    const int64_t BH = (int64_t)B * H;
+    LstmBwd a;
+    a.B = B;
+    a.H = H;
+    a.drop_scale = drop_scale();
+    for (int ph = 0; ph < L + T - 1; ++ph) {
+      a.cells = 0;
+      for (int l = L - 1; l >= 0; --l) {
+        const int t = T - 1 - (ph - (L - 1 - l));
+        if (t < 0 || t >= T) continue;
+        LstmBwdCell& c = a.cell[a.cells++];
+        c.A[0] = c.A[1] = nullptr;
+        c.W[0] = c.W[1] = nullptr;
+        c.K[0] = c.K[1] = 0;
+        c.keep = nullptr;
+        if (l + 1 < L) {  // through the input of the layer above
+          c.A[0] = gates(l + 1) + t * 4 * BH;
+          c.W[0] = wbf() + N->off_w[l + 1][0];
+          c.K[0] = 4 * H;
+          if (train_drop) c.keep = keep(l + 1) + t * BH;
+        } else if (t == T - 1) {  // from the head
+          c.A[0] = f(N->o_dy);
+          c.W[0] = wbf() + N->off_wy;
+          c.K[0] = O;
+        }
+        if (t + 1 < T) {  // from the next step
+          c.A[1] = gates(l) + (t + 1) * 4 * BH;
+          c.W[1] = wbf() + N->off_w[l][1];
+          c.K[1] = 4 * H;
+        }
+        c.c = cc(l) + (t + 1) * BH;
+        c.cprev = t > 0 ? cc(l) + t * BH : nullptr;
+        c.gates = gates(l) + t * 4 * BH;
+        c.dc = f(N->o_dc) + (size_t)l * N->Bmax * H;
+        c.first = t == T - 1;
+      }
+      LK(lstm_bwd_phase(st, a));
+    }
+    float* G = f(N->o_grad);
+    const int64_t rows = (int64_t)T * B;
+    LstmGrad g;
+    LstmSums u;
+    g.entries = u.entries = 0;
+    for (int l = 0; l < L; ++l) {
+      const float* dz = gates(l);
+      g.e[g.entries++] = {dz, l == 0 ? Xt : layer_input(l, B), G + N->off_w[l][0], rows, 4 * H, in_dim(l),
+                          4 * H, in_dim(l), 0, 0};
+      // h_{t-1}: rows of h_0 count as zero
+      g.e[g.entries++] = {dz, hh(l), G + N->off_w[l][1], rows, 4 * H, H, 4 * H, H, B, 0};
+      u.e[u.entries++] = {dz, G + N->off_w[l][2], rows, 4 * H, 0};
+    }
+    g.e[g.entries++] = {f(N->o_dy), hh(L - 1) + T * BH, G + N->off_wy, B, O, H, O, H, 0, 0};
+    u.e[u.entries++] = {f(N->o_dy), G + N->off_by, B, O, 0};
+    LK(lstm_weight_grads(st, g));
+    u.lpart = (const double*)(ws + N->o_lpart);
+    u.nlpart = lstm_head_blocks(B);
+    u.lcount = (double)B * O;
+    u.loss = f(N->o_loss);
+    LK(lstm_sums(st, u));
+    return RPOD_OK;
   }
 
   // forward over the time-major input Xt (T x B x I); y (B x O) without bias
-  template <typename TW>
-  int forward_t(const float* Xt, int B) {
+  int forward_simt(const float* Xt, int B, float* y) {
     const int H = N->H, T = N->T;
-    const TW* W = weights<TW>();
+    const float* W = f(N->o_theta);
     for (int l = 0; l < N->L; ++l) {
       const int Il = in_dim(l);
       // h_1..h_T of the layer below, masked in a training pass with dropout
       if (l > 0 && train_drop) CR2(dropout(l, B, hh(l - 1) + (size_t)B * H, xd(l)));
       const float* Xin = l == 0 ? Xt : layer_input(l, B);
       // hoisted input projection for all T steps
-      LK((gemm_ex<float, TW, float, float>(st, true, true, (int64_t)T * B, 4 * H, Il, 1, Xin, Il,
+      LK((gemm_ex<float, float, float, float>(st, true, true, (int64_t)T * B, 4 * H, Il, 1, Xin, Il,
                                                      W + N->off_w[l][0], Il, gx(l), 4 * H, 1, 0,
                                                      nullptr, false)));
       LK(cudaMemsetAsync(cc(l), 0, (size_t)B * H * 4, st));
@@ -368,7 +478,7 @@ struct Net {
       const float* bias = f(N->o_theta) + N->off_w[l][2];
       dim3 grid((B + 31) / 32, (H + 31) / 32);
       for (int t = 0; t < T; ++t) {
-        k_lstm_fwd_step<TW><<<grid, 256, 0, st>>>(B, H, gx(l) + (size_t)t * B * 4 * H, bias,
+        k_lstm_fwd_step<<<grid, 256, 0, st>>>(B, H, gx(l) + (size_t)t * B * 4 * H, bias,
                                               hh(l) + (size_t)t * B * H, W + N->off_w[l][1],
                                               cc(l) + (size_t)t * B * H, cc(l) + (size_t)(t + 1) * B * H,
                                               hh(l) + (size_t)(t + 1) * B * H,
@@ -377,8 +487,8 @@ struct Net {
       }
     }
     const float* hT = hh(N->L - 1) + (size_t)T * B * H;
-    LK((gemm_ex<float, TW, float, float>(st, true, true, B, N->O, H, 1, hT, H, W + N->off_wy, H,
-                                                   f(N->o_y), N->O, 1, 0, nullptr, false)));
+    LK((gemm_ex<float, float, float, float>(st, true, true, B, N->O, H, 1, hT, H, W + N->off_wy, H,
+                                                   y, N->O, 1, 0, nullptr, false)));
     return RPOD_OK;
   }
 
@@ -392,10 +502,9 @@ struct Net {
     return RPOD_OK;
   }
 
-  template <typename TW>
-  int backward_t(const float* Xt, int B) {
+  int backward_simt(const float* Xt, int B) {
     const int H = N->H, T = N->T, O = N->O;
-    const TW* W = weights<TW>();
+    const float* W = f(N->o_theta);
     float* G = f(N->o_grad);
     const float* hT = hh(N->L - 1) + (size_t)T * B * H;
     float* dy = f(N->o_dy);
@@ -405,7 +514,7 @@ struct Net {
     LL();
     float* dhext = f(N->o_dhext);
     LK(cudaMemsetAsync(dhext, 0, (size_t)T * B * H * 4, st));
-    LK((gemm_ex<float, TW, float, float>(st, true, false, B, H, O, 1, dy, O, W + N->off_wy, H,
+    LK((gemm_ex<float, float, float, float>(st, true, false, B, H, O, 1, dy, O, W + N->off_wy, H,
                                                    dhext + (size_t)(T - 1) * B * H, H, 1, 0, nullptr,
                                                    false)));
     float* dz = f(N->o_dz);
@@ -421,7 +530,7 @@ struct Net {
             dc, dz + (size_t)t * B * 4 * H);
         LL();
         if (t > 0)
-          LK((gemm_ex<float, TW, float, float>(st, true, false, B, H, 4 * H, 1,
+          LK((gemm_ex<float, float, float, float>(st, true, false, B, H, 4 * H, 1,
                                                          dz + (size_t)t * B * 4 * H, 4 * H,
                                                          W + N->off_w[l][1], H, dhrec, H, 1, 0, nullptr,
                                                          false)));
@@ -433,7 +542,7 @@ struct Net {
       k_colsum<<<(4 * H + 127) / 128, 128, 0, st>>>(rows, 4 * H, dz, G + N->off_w[l][2]);
       LL();
       if (l > 0) {
-        LK((gemm_ex<float, TW, float, float>(st, true, false, rows, Il, 4 * H, 1, dz, 4 * H,
+        LK((gemm_ex<float, float, float, float>(st, true, false, rows, Il, 4 * H, 1, dz, 4 * H,
                                                        W + N->off_w[l][0], Il, dhext, Il, 1, 0, nullptr,
                                                        false)));
         // the input of layer l was keep / (1 - p) times h of layer l - 1
@@ -491,11 +600,13 @@ int rpod_lstm_create(rpod_lstm** out, int32_t in_dim, int32_t hidden, int32_t la
   N->o_dhext = take(4 * T * B * maxI);
   N->o_dz = take(4 * T * B * 4 * H);
   N->o_dhrec = take(4 * B * H);
-  N->o_dc = take(4 * B * H);
+  N->o_dc = take(4 * layers * B * H);
   N->o_dx = take(4);
   N->part_floats = (size_t)32 * 4 * H * maxI;
   N->o_part = take(4 * N->part_floats);
   N->o_xd = take(4 * (size_t)(layers - 1) * T * B * H);
+  N->o_keep = take((size_t)(layers - 1) * T * B * H);
+  N->o_lpart = take(8 * (size_t)lstm_head_blocks(max_batch));
   N->o_bx = take(4 * B * T * I);
   N->o_by = take(4 * B * (size_t)out_dim);
   N->o_lsum = take(4);
@@ -558,11 +669,7 @@ int rpod_lstm_forward(rpod_lstm* N, const float* X, int32_t B, float* Y, void* w
   float* Xt = net.f(N->o_xtm);
   k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, X, Xt);
   LL();
-  if (int rc = net.forward(Xt, B)) return rc;
-  k_head_loss<<<1, 1024, 0, st>>>(B, N->O, net.f(N->o_y), net.f(N->o_theta) + N->off_by, nullptr,
-                                   nullptr, nullptr);
-  LL();
-  LK(cudaMemcpyAsync(Y, net.f(N->o_y), (size_t)4 * B * N->O, cudaMemcpyDeviceToDevice, st));
+  if (int rc = net.forward(Xt, B, Y, nullptr)) return rc;
   N->last_launches = g_launches;
   return RPOD_OK;
 }
@@ -578,10 +685,7 @@ int rpod_lstm_loss_grad(rpod_lstm* N, const float* X, const float* Yt, int32_t B
   k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, X, Xt);
   LL();
   net.train_drop = N->drop_p > 0.0 && N->L > 1;
-  if (int rc = net.forward(Xt, B)) return rc;
-  k_head_loss<<<1, 1024, 0, st>>>(B, N->O, net.f(N->o_y), net.f(N->o_theta) + N->off_by, Yt,
-                                   net.f(N->o_dy), net.f(N->o_loss));
-  LL();
+  if (int rc = net.forward(Xt, B, net.f(N->o_y), Yt)) return rc;
   if (int rc = net.backward(Xt, B)) return rc;
   if (net.train_drop) N->drop_pass += 1;
   if (loss) LK(cudaMemcpyAsync(loss, net.f(N->o_loss), 4, cudaMemcpyDefault, st));
@@ -677,10 +781,7 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
     cudaGetLastError();
   }
   for (int s = 0; s < steps; ++s) {
-    if (int rc = net.forward(cur, B)) return rc;
-    k_head_loss<<<1, 1024, 0, st>>>(B, N->O, net.f(N->o_y), net.f(N->o_theta) + N->off_by, nullptr,
-                                     nullptr, nullptr);
-    LL();
+    if (int rc = net.forward(cur, B, net.f(N->o_y), nullptr)) return rc;
     k_roll<<<blocks_for((int64_t)N->T * B * N->I), 256, 0, st>>>(B, N->T, N->I, mu_cols, cur, nxt,
                                                                  net.f(N->o_y), out, steps, s);
     LL();

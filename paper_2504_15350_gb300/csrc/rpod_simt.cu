@@ -483,7 +483,6 @@ INST_GEMM(float, float, float, float)
 INST_GEMM(float, float, float, double)
 INST_GEMM(float, double, float, float)
 INST_GEMM(double, double, double, float)
-INST_GEMM(float, __nv_bfloat16, float, float)
 #undef INST_GEMM
 
 // ------------------------------------------------------------------------
