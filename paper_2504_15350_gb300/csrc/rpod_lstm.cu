@@ -48,6 +48,8 @@ struct rpod_lstm {
   double drop_p;
   uint64_t drop_seed, drop_thr;
   int64_t drop_pass;
+  // BF16 weights: the parts of x, of every layer's h, masked h and dz, of dy
+  size_t o_px, o_ph, o_pxd, o_pz, o_pdy;
   size_t o_keep;   // dropout masks of layers 1..L-1 (bytes, as o_xd)
   size_t o_lpart;  // the head's shares of the loss
   size_t o_xd;  // masked inputs of layers 1..L-1 (T x Bmax x H each)
@@ -337,11 +339,19 @@ struct Net {
     return RPOD_OK;
   }
 
-  // y (B x O) of the time-major input Xt (T x B x I); with a target also dy and
-  // (FP32 weights) the loss.  BF16 weights: tensor-core cells, one launch per
+  // y (B x O) of the input X (element (b, t, k) at X[b sb + t stt + k]); with a
+  // target also dy and (FP32 weights) the loss.  Xt: the time-major input of
+  // the FP32-weight kernels, made from X unless X has that layout itself.  BF16 weights: tensor-core cells, one launch per
   // anti-diagonal (rpod_lstm_mma.cu); FP32 weights: the SIMT kernels here.
-  int forward(const float* Xt, int B, float* y, const float* tgt) {
-    if (!N->wfp32) return forward_mma(Xt, B, y, tgt);
+  int forward(const float* X, int64_t sb, int64_t stt, float* Xt, int B, float* y, const float* tgt) {
+    if (!N->wfp32) {
+      LK(lstm_input_parts(st, B, N->T, N->I, X, sb, stt, px()));
+      return forward_mma(B, y, tgt);
+    }
+    if (X != Xt) {
+      k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, X, Xt);
+      LL();
+    }
     CR2(forward_simt(Xt, B, y));
     k_head_loss<<<1, 1024, 0, st>>>(B, N->O, y, f(N->o_theta) + N->off_by, tgt, f(N->o_dy), f(N->o_loss));
     LL();
@@ -349,7 +359,7 @@ struct Net {
   }
   // every gradient into o_grad (BF16 weights: and the loss into o_loss)
   int backward(const float* Xt, int B) {
-    return N->wfp32 ? backward_simt(Xt, B) : backward_mma(Xt, B);
+    return N->wfp32 ? backward_simt(Xt, B) : backward_mma(B);
   }
 
   float drop_scale() const { return (float)(1.0 / (1.0 - N->drop_p)); }
@@ -357,7 +367,20 @@ struct Net {
     return (unsigned char*)(ws + N->o_keep) + (size_t)(l - 1) * N->T * N->Bmax * N->H;
   }
 
-  int forward_mma(const float* Xt, int B, float* y, const float* tgt) {
+  Parts parts(size_t o, int layer, int64_t rows, int cols) const {
+    const int ld = parts_ld(cols);
+    const int64_t plane = rows * ld;
+    return {(__nv_bfloat16*)(ws + o) + 3 * layer * plane, plane, ld};
+  }
+  int64_t prows() const { return (int64_t)N->T * N->Bmax; }
+  Parts px() const { return parts(N->o_px, 0, prows(), N->I); }
+  Parts ph(int l) const { return parts(N->o_ph, l, prows(), N->H); }         // row t B + b: h after step t
+  Parts pxd(int l) const { return parts(N->o_pxd, l - 1, prows(), N->H); }   // masked input of layer l
+  Parts pz(int l) const { return parts(N->o_pz, l, prows(), 4 * N->H); }
+  Parts pdy() const { return parts(N->o_pdy, 0, N->Bmax, N->O); }
+  Parts pin(int l) const { return l == 0 ? px() : (train_drop ? pxd(l) : ph(l - 1)); }
+
+  int forward_mma(int B, float* y, const float* tgt) {
     const int H = N->H, T = N->T, L = N->L;
     const int64_t BH = (int64_t)B * H;
     LstmFwd a;
@@ -367,70 +390,73 @@ struct Net {
     a.drop_pass = (uint64_t)N->drop_pass;
     a.drop_thr = N->drop_thr;
     a.drop_scale = drop_scale();
-    for (int ph = 0; ph < L + T - 1; ++ph) {
+    for (int d = 0; d < L + T - 1; ++d) {  // layer + time
       a.cells = 0;
       for (int l = 0; l < L; ++l) {
-        const int t = ph - l;
+        const int t = d - l;
         if (t < 0 || t >= T) continue;
         LstmFwdCell& c = a.cell[a.cells++];
         c.Il = in_dim(l);
-        c.x = l == 0 ? Xt + (size_t)t * B * N->I : layer_input(l, B) + t * BH;
-        c.hprev = t > 0 ? hh(l) + t * BH : nullptr;
+        const Parts none = {nullptr, 0, 0};
+        c.x = pin(l).rows((int64_t)t * B);
+        c.hprev = t > 0 ? ph(l).rows((int64_t)(t - 1) * B) : none;
         c.cprev = t > 0 ? cc(l) + t * BH : nullptr;
         c.Wx = wbf() + N->off_w[l][0];
         c.Wh = wbf() + N->off_w[l][1];
         c.bias = f(N->o_theta) + N->off_w[l][2];
         c.c = cc(l) + (t + 1) * BH;
-        c.h = hh(l) + (t + 1) * BH;
+        c.h = ph(l).rows((int64_t)t * B);
+        c.hf = l == L - 1 && t == T - 1 ? hh(l) : nullptr;  // for the head
         c.gates = gates(l) + t * 4 * BH;
         const bool drop = train_drop && l + 1 < L;
-        c.xd = drop ? xd(l + 1) + t * BH : nullptr;
+        c.xd = drop ? pxd(l + 1).rows((int64_t)t * B) : none;
         c.keep = drop ? keep(l + 1) + t * BH : nullptr;
         c.drop_layer = (uint64_t)(l + 1);
         c.drop_e0 = t * BH;
       }
       LK(lstm_fwd_phase(st, a));
     }
-    LK(lstm_head(st, B, N->O, H, hh(L - 1) + T * BH, wbf() + N->off_wy, f(N->o_theta) + N->off_by, y, tgt,
-                 f(N->o_dy), (double*)(ws + N->o_lpart)));
+    LK(lstm_head(st, B, N->O, H, hh(L - 1), wbf() + N->off_wy, f(N->o_theta) + N->off_by, y, tgt, pdy(),
+                 (double*)(ws + N->o_lpart)));
     return RPOD_OK;
   }
 
-  int backward_mma(const float* Xt, int B) {
+  int backward_mma(int B) {
     const int H = N->H, T = N->T, L = N->L, O = N->O;
     const int64_t BH = (int64_t)B * H;
     LstmBwd a;
     a.B = B;
     a.H = H;
     a.drop_scale = drop_scale();
-    for (int ph = 0; ph < L + T - 1; ++ph) {
+    for (int d = 0; d < L + T - 1; ++d) {  // layer + time
       a.cells = 0;
       for (int l = L - 1; l >= 0; --l) {
-        const int t = T - 1 - (ph - (L - 1 - l));
+        const int t = T - 1 - (d - (L - 1 - l));
         if (t < 0 || t >= T) continue;
         LstmBwdCell& c = a.cell[a.cells++];
-        c.A[0] = c.A[1] = nullptr;
+        c.A[0] = c.A[1] = {nullptr, 0, 0};
         c.W[0] = c.W[1] = nullptr;
         c.K[0] = c.K[1] = 0;
         c.keep = nullptr;
         if (l + 1 < L) {  // through the input of the layer above
-          c.A[0] = gates(l + 1) + t * 4 * BH;
+          c.A[0] = pz(l + 1).rows((int64_t)t * B);
           c.W[0] = wbf() + N->off_w[l + 1][0];
           c.K[0] = 4 * H;
           if (train_drop) c.keep = keep(l + 1) + t * BH;
         } else if (t == T - 1) {  // from the head
-          c.A[0] = f(N->o_dy);
+          c.A[0] = pdy();
           c.W[0] = wbf() + N->off_wy;
           c.K[0] = O;
         }
         if (t + 1 < T) {  // from the next step
-          c.A[1] = gates(l) + (t + 1) * 4 * BH;
+          c.A[1] = pz(l).rows((int64_t)(t + 1) * B);
           c.W[1] = wbf() + N->off_w[l][1];
           c.K[1] = 4 * H;
         }
         c.c = cc(l) + (t + 1) * BH;
         c.cprev = t > 0 ? cc(l) + t * BH : nullptr;
         c.gates = gates(l) + t * 4 * BH;
+        c.dz = pz(l).rows((int64_t)t * B);
         c.dc = f(N->o_dc) + (size_t)l * N->Bmax * H;
         c.first = t == T - 1;
       }
@@ -442,15 +468,13 @@ struct Net {
     LstmSums u;
     g.entries = u.entries = 0;
     for (int l = 0; l < L; ++l) {
-      const float* dz = gates(l);
-      g.e[g.entries++] = {dz, l == 0 ? Xt : layer_input(l, B), G + N->off_w[l][0], rows, 4 * H, in_dim(l),
-                          4 * H, in_dim(l), 0, 0};
-      // h_{t-1}: rows of h_0 count as zero
-      g.e[g.entries++] = {dz, hh(l), G + N->off_w[l][1], rows, 4 * H, H, 4 * H, H, B, 0};
-      u.e[u.entries++] = {dz, G + N->off_w[l][2], rows, 4 * H, 0};
+      g.e[g.entries++] = {pz(l), pin(l), G + N->off_w[l][0], rows, 4 * H, in_dim(l), 0, 0};
+      // h_{t-1}: the rows of h_0 count as zero
+      g.e[g.entries++] = {pz(l), ph(l), G + N->off_w[l][1], rows, 4 * H, H, B, 0};
+      u.e[u.entries++] = {pz(l), G + N->off_w[l][2], rows, 4 * H, 0};
     }
-    g.e[g.entries++] = {f(N->o_dy), hh(L - 1) + T * BH, G + N->off_wy, B, O, H, O, H, 0, 0};
-    u.e[u.entries++] = {f(N->o_dy), G + N->off_by, B, O, 0};
+    g.e[g.entries++] = {pdy(), ph(L - 1).rows((int64_t)(T - 1) * B), G + N->off_wy, B, O, H, 0, 0};
+    u.e[u.entries++] = {pdy(), G + N->off_by, B, O, 0};
     LK(lstm_weight_grads(st, g));
     u.lpart = (const double*)(ws + N->o_lpart);
     u.nlpart = lstm_head_blocks(B);
@@ -606,6 +630,14 @@ int rpod_lstm_create(rpod_lstm** out, int32_t in_dim, int32_t hidden, int32_t la
   N->o_part = take(4 * N->part_floats);
   N->o_xd = take(4 * (size_t)(layers - 1) * T * B * H);
   N->o_keep = take((size_t)(layers - 1) * T * B * H);
+  {
+    const size_t ldh = parts_ld(hidden), ldz = parts_ld(4 * hidden);
+    N->o_px = take(6 * T * B * parts_ld(in_dim));
+    N->o_ph = take(6 * layers * T * B * ldh);
+    N->o_pxd = take(6 * (size_t)(layers - 1) * T * B * ldh);
+    N->o_pz = take(6 * layers * T * B * ldz);
+    N->o_pdy = take(6 * B * parts_ld(out_dim));
+  }
   N->o_lpart = take(8 * (size_t)lstm_head_blocks(max_batch));
   N->o_bx = take(4 * B * T * I);
   N->o_by = take(4 * B * (size_t)out_dim);
@@ -666,10 +698,7 @@ int rpod_lstm_forward(rpod_lstm* N, const float* X, int32_t B, float* Y, void* w
   cudaStream_t st = (cudaStream_t)stream;
   Net net{N, (char*)ws, st};
   g_launches = 0;
-  float* Xt = net.f(N->o_xtm);
-  k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, X, Xt);
-  LL();
-  if (int rc = net.forward(Xt, B, Y, nullptr)) return rc;
+  if (int rc = net.forward(X, (int64_t)N->T * N->I, N->I, net.f(N->o_xtm), B, Y, nullptr)) return rc;
   N->last_launches = g_launches;
   return RPOD_OK;
 }
@@ -682,10 +711,8 @@ int rpod_lstm_loss_grad(rpod_lstm* N, const float* X, const float* Yt, int32_t B
   Net net{N, (char*)ws, st};
   g_launches = 0;
   float* Xt = net.f(N->o_xtm);
-  k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, X, Xt);
-  LL();
   net.train_drop = N->drop_p > 0.0 && N->L > 1;
-  if (int rc = net.forward(Xt, B, net.f(N->o_y), Yt)) return rc;
+  if (int rc = net.forward(X, (int64_t)N->T * N->I, N->I, Xt, B, net.f(N->o_y), Yt)) return rc;
   if (int rc = net.backward(Xt, B)) return rc;
   if (net.train_drop) N->drop_pass += 1;
   if (loss) LK(cudaMemcpyAsync(loss, net.f(N->o_loss), 4, cudaMemcpyDefault, st));
@@ -781,7 +808,7 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
     cudaGetLastError();
   }
   for (int s = 0; s < steps; ++s) {
-    if (int rc = net.forward(cur, B, net.f(N->o_y), nullptr)) return rc;
+    if (int rc = net.forward(cur, N->I, (int64_t)B * N->I, cur, B, net.f(N->o_y), nullptr)) return rc;
     k_roll<<<blocks_for((int64_t)N->T * B * N->I), 256, 0, st>>>(B, N->T, N->I, mu_cols, cur, nxt,
                                                                  net.f(N->o_y), out, steps, s);
     LL();
