@@ -63,6 +63,30 @@ __device__ __forceinline__ void philox4x64_10(uint64_t c[4], uint64_t k0, uint64
 extern thread_local int g_launches;
 inline void note_launch() { ++g_launches; }
 
+// Launch that may begin before the kernel in front of it on the stream has
+// ended: its CTAs are placed and run up to pdl_wait(), which every kernel
+// launched this way calls before it touches anything that an earlier kernel
+// writes or reads.  pdl_trigger(), at a kernel's start, lets the next one in.  A
+// kernel without pdl_wait() is launched with <<<>>> and starts after all in
+// front of it have ended.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*fn)(P...), A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  note_launch();
+  return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // ---- generic SIMT GEMM --------------------------------------------------
 // C_z = sum_{k in split z} A(i, k) B(k, j) for i < M, j < N,
 //   A(i, k) = a_kcontig ? A[k + i*lda] : A[i + k*lda]

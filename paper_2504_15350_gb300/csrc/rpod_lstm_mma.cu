@@ -223,18 +223,22 @@ __global__ void __launch_bounds__(256, 2) k_cell_fwd(const __grid_constant__ Lst
       rb[i] = ld_pair<EVEN>(pw + (int64_t)((i & 3) * H + (i >> 2) * 8) * K,
                             k < K && u0 + (i >> 2) * 8 + warp < H, k + 1 < K);
   };
-  load_a(0);
-  load_a(1);
+  pdl_trigger();
   uint32_t rb0[NB], rb1[NB];
-  load_w(0, rb0);
+  load_w(0, rb0);  // the weights are older than this pass
   load_w(1, rb1);
   // what the epilogue reads: rows (lane >> 2) + 8 h, units 2 (lane & 3) + j
   const int eb = b0 + wm * 16 + (lane >> 2), eu = u0 + wn * 8 + 2 * (lane & 3);
   float bias[4][2], cp[2][2];
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
     for (int q = 0; q < 4; ++q) bias[q][j] = eu + j < H ? C.bias[q * H + eu + j] : 0.f;
+  pdl_wait();
+  load_a(0);
+  load_a(1);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
 #pragma unroll
     for (int h = 0; h < 2; ++h)
       cp[h][j] = (C.cprev && eb + 8 * h < B && eu + j < H) ? C.cprev[(int64_t)(eb + 8 * h) * H + eu + j] : 0.f;
@@ -351,11 +355,13 @@ __global__ void __launch_bounds__(256, 2) k_cell_bwd(const __grid_constant__ Lst
     for (int i = 0; i < NB; ++i)
       rb[i] = ld_pair<EVEN>(pw + i * KR * H, u0 + bu < H && kw + i * KR < K, u0 + bu + 1 < H);
   };
+  pdl_trigger();
+  uint32_t rb0[NB], rb1[NB];
+  load_w(0, rb0);  // the weights are older than this pass
+  load_w(1, rb1);
+  pdl_wait();
   load_a(0);
   load_a(1);
-  uint32_t rb0[NB], rb1[NB];
-  load_w(0, rb0);
-  load_w(1, rb1);
   Acc acc;
   acc.clear();
   auto chunk = [&](int ch, uint32_t (&rb)[NB], __nv_bfloat16 (&Bs)[64][UN + 8]) {
@@ -456,6 +462,7 @@ struct GradStage {
 __global__ void __launch_bounds__(256, 2) k_weight_grads(const __grid_constant__ LstmGrad a) {
   extern __shared__ __align__(16) uint8_t sm[];
   GradStage* const stg = (GradStage*)sm;
+  pdl_trigger();
   int ei = 0;
   while (ei + 1 < a.entries && (int)blockIdx.x >= a.e[ei + 1].tile0) ++ei;
   const LstmGradEntry& E = a.e[ei];
@@ -474,6 +481,7 @@ __global__ void __launch_bounds__(256, 2) k_weight_grads(const __grid_constant__
   };
   Acc acc;
   acc.clear();
+  pdl_wait();
   load(0, stg[0]);
   for (int64_t k0 = 0; k0 < K; k0 += 64) {
     GradStage& S = stg[(k0 >> 6) & 1];
@@ -523,6 +531,8 @@ __global__ void __cluster_dims__(1, kSumSplit, 1) __launch_bounds__(1024) k_lstm
   __shared__ double tot[64];
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if ((int)blockIdx.x == a.blocks) {
     if (threadIdx.x == 0 && blockIdx.y == 0) {
@@ -575,6 +585,7 @@ __global__ void __cluster_dims__(1, kSumSplit, 1) __launch_bounds__(1024) k_lstm
 
 // ---- parts of the windows
 __global__ void k_input_parts(int B, int T, int I, const float* __restrict__ X, int64_t sb, int64_t stt, Parts out) {
+  pdl_trigger();
   const int64_t row = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= (int64_t)T * B) return;
   const float* x = X + (row % B) * sb + (row / B) * stt;
@@ -587,6 +598,8 @@ __global__ void __launch_bounds__(kHeadRows * 32)
 k_head(int B, int O, int H, const float* __restrict__ h, const __nv_bfloat16* __restrict__ Wy,
        const float* __restrict__ by, float* __restrict__ y, const float* __restrict__ tgt,
        const Parts dy, double* __restrict__ lpart) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ double red[kHeadRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kHeadRows + warp;
@@ -648,9 +661,8 @@ cudaError_t fwd_launch(cudaStream_t st, const LstmFwd& a) {
   static_assert(smem >= (WK - 1) * WM * WN * 2048, "the shares fit");
   cudaError_t e = cudaFuncSetAttribute(k_cell_fwd<WM, WN, WK, EVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_cell_fwd<WM, WN, WK, EVEN><<<dim3((a.B + BM - 1) / BM, (a.H + UN - 1) / UN, a.cells), 256, smem, st>>>(a);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(st, dim3((a.B + BM - 1) / BM, (a.H + UN - 1) / UN, a.cells), 256, smem,
+                    k_cell_fwd<WM, WN, WK, EVEN>, a);
 }
 template <int WM, int WN, int WK, bool EVEN>
 cudaError_t bwd_launch(cudaStream_t st, const LstmBwd& a) {
@@ -664,13 +676,15 @@ cudaError_t bwd_launch(cudaStream_t st, const LstmBwd& a) {
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 1;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 2;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_pdl
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, k_cell_bwd<WM, WN, WK, EVEN>, a);
   note_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
@@ -700,9 +714,7 @@ cudaError_t lstm_weight_grads(cudaStream_t st, LstmGrad& a) {
   const int smem = 2 * (int)sizeof(GradStage);
   const cudaError_t e = cudaFuncSetAttribute(k_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_weight_grads<<<a.tiles, 256, smem, st>>>(a);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(st, a.tiles, 256, smem, k_weight_grads, a);
 }
 
 cudaError_t lstm_sums(cudaStream_t st, LstmSums& a) {
@@ -711,9 +723,7 @@ cudaError_t lstm_sums(cudaStream_t st, LstmSums& a) {
     a.e[i].block0 = a.blocks;
     a.blocks += (a.e[i].N + 63) / 64;
   }
-  k_lstm_sums<<<dim3(a.blocks + 1, kSumSplit), 1024, 0, st>>>(a);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(st, dim3(a.blocks + 1, kSumSplit), 1024, 0, k_lstm_sums, a);
 }
 
 cudaError_t lstm_input_parts(cudaStream_t st, int B, int T, int I, const float* X, int64_t sb, int64_t stt,
@@ -727,9 +737,7 @@ int lstm_head_blocks(int B) { return (B + kHeadRows - 1) / kHeadRows; }
 
 cudaError_t lstm_head(cudaStream_t st, int B, int O, int H, const float* h, const __nv_bfloat16* Wy,
                       const float* by, float* y, const float* tgt, Parts dy, double* lpart) {
-  k_head<<<lstm_head_blocks(B), kHeadRows * 32, 0, st>>>(B, O, H, h, Wy, by, y, tgt, dy, lpart);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(st, lstm_head_blocks(B), kHeadRows * 32, 0, k_head, B, O, H, h, Wy, by, y, tgt, dy, lpart);
 }
 
 }  // namespace rpod
