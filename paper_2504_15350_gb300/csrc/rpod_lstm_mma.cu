@@ -89,6 +89,27 @@ struct Acc {
         hi[n][i] = lo[n][i] = 0.f;
       }
   }
+  // The same with the rounding error of each sum (Knuth's TwoSum) kept with the
+  // small products, for the weight gradients' many chunks: with plain sums the 80
+  // of window 10, batch 512 left 1.3e-7 of error against 64 bits, now 1.1e-7, that
+  // of FP32 products.  finish() adds what is left.
+  __device__ __forceinline__ void flush_exact() {
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float s = sum[n][i], y = hi[n][i] + lo[n][i], t = s + y, b = t - s;
+        lo[n][i] = (s - (t - b)) + (y - b);
+        sum[n][i] = t;
+        hi[n][i] = 0.f;
+      }
+  }
+  __device__ __forceinline__ void finish() {
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sum[n][i] += lo[n][i];
+  }
 };
 
 // 16 x 32 x 16: FP32 operand in three parts times BF16, n-tile n's two registers
@@ -510,8 +531,9 @@ __global__ void __launch_bounds__(256, 2) k_weight_grads(const __grid_constant__
                      fx[px[t]][2 * n2 + 1]);
       }
     }
-    acc.flush();
+    acc.flush_exact();
   }
+  acc.finish();
 #pragma unroll
   for (int n = 0; n < 4; ++n)
 #pragma unroll
