@@ -33,46 +33,98 @@ template <> __device__ __forceinline__ __half cvt<__half>(double x) { return __d
 // Entry e = i + j m of Lambda is z0 (e even) or z1 (e odd) of the
 // Box-Muller pair of Philox block e / 2: u1 = (w0 >> 11 + 1) 2^-53,
 // u2 = (w1 >> 11) 2^-53, z0 = sqrt(-2 ln u1) cos(2 pi u2), z1 = ... sin.
-// FP64 and FP32 sketches evaluate it in FP64.  A sketch stored in a 16-bit
-// type keeps 8 or 11 mantissa bits, so it is evaluated in FP32 (GB300's FP64
-// transcendental throughput made the FP64 form of this kernel 90 us for
-// m l = 1.2e6): the integer words and uniforms are the same, ln u1 is taken
+// An FP64 sketch evaluates it in FP64.  GB300 issues about two FP64 operations
+// a clock and SM, so the other forms take no FP64 operation, conversions
+// included: 60 x 64000 entries in FP32 262 -> 38 us, 85 x 90225 in BF16
+// 64 -> 60 us, most of it now the 64-bit multiplications of Philox.
+//
+// FP32 sketch: values as unevaluated sums of two FP32 numbers, relative error
+// below 2^-32 before the one rounding to FP32, so that an entry differs from
+// the rounded FP64 value only within 2^-8 ulp of a rounding boundary.
+// ln: u1 = 2^e f with f in [2^-1/2, 2^1/2), ln f = 2 atanh((f - 1) / (f + 1)),
+// numerator and denominator exact integers, Taylor series.  sin and cos: u2 split
+// into quarter turns and a remainder in integers, Taylor series of sin(pi f)
+// and cos(pi f), |f| <= 1/4.
+//
+// 16-bit sketch (8 or 11 mantissa bits kept): evaluated in FP32.  ln u1 is taken
 // as log1p(-(1 - u1)) for u1 >= 1/2 so that u1 near 1 keeps its relative
 // accuracy, and the result differs from the FP64 value by a few FP32 ulps,
 // which changes the 16-bit rounding only for values within that distance
 // of a rounding boundary (the angle is reduced to within a quarter turn in
 // integer arithmetic, so values near the zeros of sin and cos keep their
 // relative accuracy).
+struct F2 {
+  float h, l;
+};
+// a + b for |a| >= |b| or a = 0 (Fast2Sum), and for any a, b (TwoSum)
+__device__ __forceinline__ F2 sum_fast(float a, float b) {
+  const float s = a + b;
+  return {s, b - (s - a)};
+}
+__device__ __forceinline__ F2 sum_two(float a, float b) {
+  const float s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+__device__ __forceinline__ F2 prod2(F2 a, F2 b) {
+  const float p = __fmul_rn(a.h, b.h);  // never contracted into a sum that is corrected by it
+  return {p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h)};
+}
+// c + x for |c.h| >= |x.h|
+__device__ __forceinline__ F2 add2(F2 c, F2 x) {
+  const F2 s = sum_fast(c.h, x.h);
+  return {s.h, s.l + (c.l + x.l)};
+}
+__device__ __forceinline__ F2 from_int(int64_t v) {
+  const float h = (float)v;
+  return {h, (float)(v - (int64_t)h)};
+}
+
+// sqrt(-2 ln((x0 + 1) 2^-53)), x0 < 2^53
+__device__ __forceinline__ F2 bm_radius(uint64_t x0) {
+  const uint64_t n = x0 + 1;
+  const int lz = __clzll((long long)n);  // 10 or more
+  const int64_t M = (int64_t)((n << lz) >> 3);  // f 2^60, exact, 1 <= f < 2
+  const bool up = (uint32_t)(M >> 29) > 0xB504F333u;  // f > 2^1/2: f / 2 and e + 1
+  const int e = 10 - lz + (up ? 1 : 0);
+  const int64_t one = up ? 1ll << 61 : 1ll << 60;
+  const F2 a = from_int(M - one), d = from_int(M + one);
+  // s = a / d
+  const float q = __fdividef(a.h, d.h);
+  const F2 s{q, __fdividef(fmaf(-q, d.h, a.h) + (a.l - q * d.l), d.h)};
+  const F2 z = prod2(s, s);  // <= 0.0295
+  // ln f = 2 s (1 + z / 3 + z^2 / 5 + ...)
+  const float w = z.h * (0.2f + z.h * ((1.f / 7) + z.h * ((1.f / 9) + z.h * ((1.f / 11) + z.h * ((1.f / 13) + z.h * (1.f / 15))))));
+  const F2 t = prod2(z, add2({0x1.555556p-2f, -0x1.555556p-27f}, {w, 0.f}));
+  const F2 lf = add2(s, prod2(s, t));
+  // -2 ln u1 = -4 lf - 2 e ln 2; the 15 upper bits of ln 2 times e are exact
+  const float e2 = -2.f * (float)e;
+  const F2 x = sum_two(e2 * 0x1.62e4p-1f, -4.f * lf.h);
+  const F2 y = sum_fast(x.h, x.l + fmaf(e2, 0x1.7f7d1cp-20f, -4.f * lf.l));
+  const float r = sqrtf(y.h);
+  return {r, r > 0.f ? __fdividef(fmaf(-r, r, y.h) + y.l, 2.f * r) : 0.f};
+}
+
+// sin and cos of pi f for f = k 2^-52, |f| <= 1/4
+__device__ __forceinline__ void bm_sincos(int64_t k, F2& sn, F2& cs) {
+  F2 f = from_int(k);
+  f.h *= 0x1p-52f;
+  f.l *= 0x1p-52f;
+  const F2 z = prod2(f, f);
+  const float ws = z.h * (-0x1.32d2ccp-1f + z.h * (0x1.507834p-4f + z.h * (-0x1.e30750p-8f + z.h * 0x1.e8f434p-12f)));
+  F2 p = add2({0x1.466bc6p+1f, 0x1.dd6ab8p-25f}, {ws, 0.f});
+  p = add2({-0x1.4abbcep+2f, -0x1.896f94p-24f}, prod2(p, z));
+  p = add2({0x1.921fb6p+1f, -0x1.777a5cp-24f}, prod2(p, z));
+  sn = prod2(f, p);
+  const float wc = z.h * (-0x1.55d3c8p+0f + z.h * (0x1.e1f506p-3f + z.h * (-0x1.a6d1f2p-6f + z.h * (0x1.f9d38ap-10f - z.h * 0x1.b6e250p-14f))));
+  F2 c = add2({0x1.03c1f0p+2f, 0x1.036b58p-23f}, {wc, 0.f});
+  c = add2({-0x1.3bd3ccp+2f, -0x1.37c8bcp-23f}, prod2(c, z));
+  cs = add2({1.f, 0.f}, prod2(c, z));
+}
+
 template <typename T>
 __device__ __forceinline__ void box_muller_store(uint64_t w0, uint64_t w1, T* a, T* b) {
   const uint64_t x0 = w0 >> 11, x1 = w1 >> 11;
-  if constexpr (sizeof(T) == 2) {
-    float lnu;
-    if (x0 >= (1ull << 52)) {
-      // 1 - u1 = (2^53 - 1 - x0) 2^-53, exact in FP64, accurate in FP32
-      const float d = (float)((double)((1ull << 53) - 1ull - x0) * 0x1p-53);
-      lnu = log1pf(-d);
-    } else {
-      lnu = logf((float)(((double)x0 + 1.0) * 0x1p-53));
-    }
-    const float r = sqrtf(-2.f * lnu);
-    // angle pi t with t = x1 2^-52 in [0, 2): split t = q/2 + f exactly in
-    // integers (|f| <= 1/4) so that sin and cos keep their relative accuracy
-    // near their zeros, then rotate by the quarter turns q
-    const int64_t q = (int64_t)((x1 + (1ull << 50)) >> 51);
-    const float f = (float)((double)((int64_t)x1 - q * (int64_t)(1ull << 51)) * 0x1p-52);
-    float s0, c0;
-    sincospif(f, &s0, &c0);
-    float sn, cs;
-    switch (q & 3) {
-      case 0: sn = s0; cs = c0; break;
-      case 1: sn = c0; cs = -s0; break;
-      case 2: sn = -s0; cs = -c0; break;
-      default: sn = -c0; cs = s0; break;
-    }
-    *a = cvt<T>(r * cs);
-    if (b) *b = cvt<T>(r * sn);
-  } else {
+  if constexpr (sizeof(T) == 8) {
     const double u1 = ((double)x0 + 1.0) * 0x1p-53;
     const double u2 = (double)x1 * 0x1p-53;
     const double r = sqrt(-2.0 * log(u1));
@@ -80,6 +132,36 @@ __device__ __forceinline__ void box_muller_store(uint64_t w0, uint64_t w1, T* a,
     sincospi(2.0 * u2, &sn, &cs);
     *a = cvt<T>(r * cs);
     if (b) *b = cvt<T>(r * sn);
+  } else {
+    // angle pi t with t = x1 2^-52 in [0, 2): split t = q/2 + f exactly in
+    // integers (|f| <= 1/4) so that sin and cos keep their relative accuracy
+    // near their zeros, then rotate by the quarter turns q
+    const int64_t q = (int64_t)((x1 + (1ull << 50)) >> 51);
+    const int64_t k = (int64_t)x1 - q * (int64_t)(1ull << 51);
+    float zc, zs;  // r cos(pi f), r sin(pi f)
+    if constexpr (sizeof(T) == 4) {
+      const F2 r = bm_radius(x0);
+      F2 sn, cs;
+      bm_sincos(k, sn, cs);
+      const F2 c = prod2(r, cs), s = prod2(r, sn);
+      zc = c.h + c.l;
+      zs = s.h + s.l;
+    } else {
+      float lnu;
+      if (x0 >= (1ull << 52))
+        lnu = log1pf(-((float)(int64_t)((1ull << 53) - 1ull - x0) * 0x1p-53f));  // 1 - u1, exact before the rounding
+      else
+        lnu = logf((float)(int64_t)(x0 + 1) * 0x1p-53f);
+      const float r = sqrtf(-2.f * lnu);
+      float s0, c0;
+      sincospif((float)k * 0x1p-52f, &s0, &c0);
+      zc = r * c0;
+      zs = r * s0;
+    }
+    // a quarter turn on: (cos, sin) -> (-sin, cos)
+    const float ca = (q & 1) ? zs : zc, sa = (q & 1) ? zc : zs;
+    *a = cvt<T>(((q + 1) & 2) ? -ca : ca);
+    if (b) *b = cvt<T>((q & 2) ? -sa : sa);
   }
 }
 
