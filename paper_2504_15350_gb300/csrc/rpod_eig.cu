@@ -28,7 +28,7 @@
 //      threads per eigenvalue, in different warps: one runs the forward
 //      recurrences, one the backward ones.
 //   3. (one CTA) Vectors of eigenvalues closer than 1e-5 ||T|| are
-//      orthogonalised against each other (Gram-Schmidt in ascending order);
+//      orthogonalised against each other (Gram-Schmidt from the largest down);
 //      a vector that loses more than half its norm there (a multiple
 //      eigenvalue) is replaced by inverse iteration with T - lambda I from
 //      a pseudo-random vector, orthogonalised against the cluster's other
@@ -61,17 +61,14 @@ constexpr int kEpb = 8;            // eigenvalues per CTA of that kernel
 constexpr int kBackThreads = 256;  // back-transformation: 16 column pairs per CTA
 constexpr int kBackCols = 32;
 
-// Rows of A start on 16-byte boundaries; the cluster pass's Z uses a leading
-// dimension of 1 mod 32, so that a column and a row each fall in distinct
-// banks.
+// Rows of A start on 16-byte boundaries.
 __host__ __device__ inline int eig_lda(int l) { return (l + 3) & ~3; }
-__host__ __device__ inline int eig_ldx(int l) { return ((l + 31) & ~31) + 1; }
 
 // Shared memory of the tridiagonalization (A, reflector and p buffers, d, e,
-// tau), the cluster pass (Z and the dot-product buffer) and the
+// tau), the cluster pass (the finished vectors) and the
 // back-transformation (the reflector rows).
 size_t tri_smem_bytes(int l) { return sizeof(float) * ((size_t)l * eig_lda(l) + 7 * (size_t)kMaxL); }
-size_t clu_smem_bytes(int l) { return sizeof(float) * ((size_t)l * eig_ldx(l) + (size_t)kMaxL); }
+size_t clu_smem_bytes(int l) { return sizeof(float) * (size_t)l * kMaxL; }
 size_t back_smem_bytes(int l) { return sizeof(float) * (size_t)l * eig_lda(l); }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -504,215 +501,235 @@ k_eig_vec(int l, const float* __restrict__ sd, const float* __restrict__ se, flo
   if (tid < kEpb && g0 + tid < l) slam[g0 + tid] = lam[tid];
 }
 
+// A vector of a multiple eigenvalue lam_a by one warp: two steps of inverse
+// iteration with T - lam_a I from a pseudo-random vector (the invariant subspace
+// of the eigenvalues near lam_a grows by about 1/eps against every other
+// eigenvector).  The recurrences run on one lane with their state in registers
+// and the pivots' reciprocals taken beforehand by all lanes: with both in shared
+// memory a vector took about 22 us.
+struct InvIter {
+  float4 lu[kMaxL];  // multiplier, U's diagonal's reciprocal and two superdiagonals
+  float v[kMaxL], d[kMaxL];
+  int piv[kMaxL];
+};
+__device__ void inverse_iteration(InvIter& s, int l, int a, const float* dd, const float* ee,
+                                  const float* lam, float (&x)[4]) {
+  const int lane = threadIdx.x & 31;
+  const float lm = lam[a];
+  const float tn = fmaxf(fmaxf(fabsf(lam[0]), fabsf(lam[l - 1])), 1e-30f);
+  const float tiny = FLT_EPSILON * tn;
+  for (int r = lane; r < l; r += 32) {
+    const uint32_t hsh = mix32((uint32_t)(a * 131 + r) * 2654435761u + 12345u);
+    s.v[r] = (float)(hsh >> 8) * (1.f / 8388608.f) - 1.f;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    // LU with partial pivoting; cd, cu: the current row's diagonal and superdiagonal
+    float cd = dd[0] - lm, cu = l > 1 ? ee[0] : 0.f;
+#pragma unroll 4
+    for (int k = 0; k + 1 < l; ++k) {
+      const float el = ee[k], nd = dd[k + 1] - lm, nu = k + 2 < l ? ee[k + 1] : 0.f;
+      if (fabsf(cd) >= fabsf(el)) {
+        if (!(fabsf(cd) >= tiny)) cd = cd < 0.f ? -tiny : tiny;
+        const float f = el / cd;
+        s.d[k] = cd;
+        s.lu[k] = make_float4(f, 0.f, cu, 0.f);
+        s.piv[k] = 0;
+        cd = nd - f * cu;
+        cu = nu;
+      } else {
+        const float f = cd / el;
+        s.d[k] = el;
+        s.lu[k] = make_float4(f, 0.f, nd, nu);
+        s.piv[k] = 1;
+        cd = cu - f * nd;
+        cu = -f * nu;
+      }
+    }
+    s.d[l - 1] = cd;
+    s.lu[l - 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __syncwarp();
+  // pivots below eps ||T|| are raised to it (a perturbation of T at rounding
+  // level) so the solves cannot overflow
+  for (int k = lane; k < l; k += 32) {
+    float d = s.d[k];
+    if (!(fabsf(d) >= tiny)) d = d < 0.f ? -tiny : tiny;
+    s.lu[k].y = 1.f / d;
+  }
+  __syncwarp();
+  for (int step = 0; step < 2; ++step) {
+    float mx = 0.f;
+    if (lane == 0) {
+      float y = s.v[0];
+#pragma unroll 4
+      for (int k = 0; k + 1 < l; ++k) {
+        const float f = s.lu[k].x, nx = s.v[k + 1];
+        const bool pv = s.piv[k] != 0;
+        s.v[k] = pv ? nx : y;
+        y = pv ? y - f * nx : nx - f * y;
+      }
+      s.v[l - 1] = y;
+      float v1 = 0.f, v2 = 0.f;
+#pragma unroll 4
+      for (int k = l - 1; k >= 0; --k) {
+        const float4 u = s.lu[k];
+        const float v = (s.v[k] - u.w * v2 - u.z * v1) * u.y;
+        s.v[k] = v;
+        mx = fmaxf(mx, fabsf(v));
+        v2 = v1;
+        v1 = v;
+      }
+    }
+    mx = __shfl_sync(0xffffffffu, mx, 0);
+    __syncwarp();
+    const float sc = mx > 0.f && mx <= FLT_MAX ? 1.f / mx : 0.f;
+    for (int k = lane; k < l; k += 32) s.v[k] = sc > 0.f ? s.v[k] * sc : (k == a ? 1.f : 0.f);
+    __syncwarp();
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) x[u] = lane + 32 * u < l ? s.v[lane + 32 * u] : 0.f;
+}
+
+// x_v -= (q . x_v) q for a warp's first NV vectors, those of index >= start
+// (vector v has index warp + 32 v)
+template <int NV>
+__device__ __forceinline__ void take_out(float (&x)[4][4], const float (&q)[4], int warp, int start) {
+  float d[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    d[v] = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) d[v] = fmaf(q[u], x[v][u], d[v]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) d[v] += __shfl_xor_sync(0xffffffffu, d[v], o);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    if (warp + 32 * v < start) d[v] = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[v][u] = fmaf(-d[v], q[u], x[v][u]);
+  }
+}
+
 // Step 3: vectors of clustered eigenvalues (Z in place); without a cluster
 // the kernel ends after the gap test.
+//
+// The vectors of close eigenvalues are orthogonalised, the largest of a cluster
+// first: the gap test is absolute, so the small end of a graded spectrum is
+// one cluster, and its larger eigenvalues' vectors are accurate where the
+// smallest ones', below the rounding of T, are noise that must not be
+// subtracted from them.  A finished vector is taken out of all smaller ones of
+// its cluster at once (modified Gram-Schmidt): every vector stays in the
+// registers of one warp, and a step is one shared row, one barrier and one dot
+// product per vector.  One pass is enough, since a vector that loses more than
+// half its norm (a multiple eigenvalue) is replaced: by inverse iteration,
+// which keeps the replacement in its own cluster's invariant subspace
+// (orthogonalising a random vector against all other vectors does not: while
+// another cluster still holds a duplicate, that complement mixes both clusters'
+// missing directions), then two passes of modified Gram-Schmidt against the
+// cluster's finished vectors.
+//
+// Bound: the chain of steps, one CTA.  Measured at l = 85 with the noise end of the
+// spectrum as one cluster: basis of 8192 x 90225 3212 -> 3017 us (234 us of it
+// were this kernel, with two classical passes of four barriers per vector).
 __global__ void __launch_bounds__(kEigThreads)
 k_eig_cluster(int l, const float* __restrict__ sd, const float* __restrict__ se,
               const float* __restrict__ slam, float* __restrict__ Z, unsigned* __restrict__ status) {
+  static_assert(kMaxL == 128 && kEigThreads == 1024, "four vectors of four values a lane");
   extern __shared__ float4 sm4[];
-  const int ldx = eig_ldx(l);
-  float* const Xs = reinterpret_cast<float*>(sm4);  // Z: row r at r * ldx
-  float* const Ws = Xs + (size_t)l * ldx;           // dot products
+  float* const Q = reinterpret_cast<float*>(sm4);  // finished vector g at g * kMaxL
   __shared__ float lam[kMaxL], dd[kMaxL], ee[kMaxL];
-  __shared__ int s_any;
+  __shared__ int s_any, s_rep;
+  __shared__ InvIter s_inv;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
-  if (tid == 0) s_any = 0;
+  if (tid == 0) s_any = s_rep = 0;
   for (int k = tid; k < l; k += nt) {
     lam[k] = slam[k];
     dd[k] = sd[k];
     ee[k] = se[k];
   }
   __syncthreads();
-  {
-    const float ctol = fmaxf(1e-5f * fmaxf(fabsf(lam[0]), fabsf(lam[l - 1])), 1e-15f);
-    for (int i = tid + 1; i < l; i += nt)
-      if (lam[i] - lam[i - 1] <= ctol) s_any = 1;
-  }
+  // eigenvalues closer than 1e-15 are one cluster even in a (near) zero matrix
+  const float ctol = fmaxf(1e-5f * fmaxf(fabsf(lam[0]), fabsf(lam[l - 1])), 1e-15f);
+  for (int i = tid + 1; i < l; i += nt)
+    if (lam[i] - lam[i - 1] <= ctol) s_any = 1;
   __syncthreads();
   if (!s_any) {
     if (tid == 0) status[4] = 0u;
     return;
   }
-  for (int e = tid; e < l * l; e += nt) {
-    const int g = e / l, r = e - g * l;
-    Xs[r * ldx + g] = Z[e];
-  }
-  __syncthreads();
-  // orthogonalise vectors of close eigenvalues, the largest of a cluster
-  // first: the gap test is absolute, so the small end of a graded spectrum
-  // is one cluster, and its larger eigenvalues' vectors are accurate where
-  // the smallest ones', below the rounding of T, are noise that must not be
-  // subtracted from them.  Per vector a of a
-  // cluster, two classical Gram-Schmidt passes against the cluster's
-  // vectors above a (already orthonormal): the dots by one warp each, the
-  // update by 16 threads per row.  A vector that loses more than half its
-  // norm (a multiple eigenvalue) is replaced by warp 0: inverse iteration
-  // with T - lambda I from a pseudo-random vector, which keeps the
-  // replacement in its own cluster's invariant subspace (orthogonalising a
-  // random vector against all other vectors does not: while another
-  // cluster still holds a duplicate, that complement mixes both clusters'
-  // missing directions), then modified Gram-Schmidt against the cluster's
-  // processed vectors.  The forward-pivot array is free again and holds the
-  // dot products.
-  {
-    float* const dts = Ws;
-    __shared__ float s_n2;
-    // inverse iteration of a replaced vector: LU of T - lambda I and the vector
-    __shared__ float s_d[kMaxL], s_du[kMaxL], s_dl[kMaxL], s_du2[kMaxL], s_iv[kMaxL];
-    __shared__ int s_piv[kMaxL];
-    // eigenvalues closer than 1e-15 are one cluster even in a (near) zero matrix
-    const float ctol = fmaxf(1e-5f * fmaxf(fabsf(lam[0]), fabsf(lam[l - 1])), 1e-15f);
-    const int part = tid & 15, rsub = tid >> 4;
-    const unsigned hmask = 0xFFFFu << (lane & 16);
-    int start = 0, nrep = 0;
-    for (int i = 1; i <= l; ++i) {
-      if (i < l && lam[i] - lam[i - 1] <= ctol) continue;
-      for (int a = i - 2; a >= start; --a) {
-        for (int pass = 0; pass < 2; ++pass) {
-          for (int b = a + 1 + warp; b < i; b += nt >> 5) {
-            float dt = 0.f;
-            for (int r = lane; r < l; r += 32) dt = fmaf(Xs[r * ldx + b], Xs[r * ldx + a], dt);
-            dt = warp_sum(dt);
-            if (lane == 0) dts[b] = dt;
-          }
-          __syncthreads();
-          for (int r0 = 0; r0 < l; r0 += nt >> 4) {
-            const int r = r0 + rsub;
-            float acc = 0.f;
-            if (r < l)
-              for (int b = a + 1 + part; b < i; b += 16) acc = fmaf(dts[b], Xs[r * ldx + b], acc);
-            acc += __shfl_xor_sync(hmask, acc, 1);
-            acc += __shfl_xor_sync(hmask, acc, 2);
-            acc += __shfl_xor_sync(hmask, acc, 4);
-            acc += __shfl_xor_sync(hmask, acc, 8);
-            if (r < l && part == 0) Xs[r * ldx + a] -= acc;
-          }
-          __syncthreads();
-        }
-        if (warp == 0) {
-          float n2 = 0.f;
-          for (int r = lane; r < l; r += 32) n2 = fmaf(Xs[r * ldx + a], Xs[r * ldx + a], n2);
-          n2 = warp_sum(n2);
-          if (n2 < 0.25f) {
-            // a multiple eigenvalue: two steps of inverse iteration with
-            // T - lambda_a I from a pseudo-random vector (the cluster's own
-            // invariant subspace grows by about 1/eps against every other
-            // eigenvector), then Gram-Schmidt against the cluster's
-            // processed vectors
-            ++nrep;
-            const float lm = lam[a];
-            for (int r = lane; r < l; r += 32) {
-              const uint32_t hsh = mix32((uint32_t)(a * 131 + r) * 2654435761u + 12345u);
-              s_iv[r] = (float)(hsh >> 8) * (1.f / 8388608.f) - 1.f;
-            }
-            __syncwarp();
-            if (lane == 0) {
-              // LU with partial pivoting of the tridiagonal T - lm I
-              const float tn = fmaxf(fmaxf(fabsf(lam[0]), fabsf(lam[l - 1])), 1e-30f);
-              const float tiny = FLT_EPSILON * tn;
-              for (int k = 0; k < l; ++k) {
-                s_d[k] = dd[k] - lm;
-                s_du[k] = k + 1 < l ? ee[k] : 0.f;
-                s_dl[k] = k + 1 < l ? ee[k] : 0.f;
-                s_du2[k] = 0.f;
-                s_piv[k] = 0;
-              }
-              for (int k = 0; k + 1 < l; ++k) {
-                if (fabsf(s_d[k]) >= fabsf(s_dl[k])) {
-                  if (!(fabsf(s_d[k]) >= tiny)) s_d[k] = s_d[k] < 0.f ? -tiny : tiny;
-                  const float f = s_dl[k] / s_d[k];
-                  s_dl[k] = f;
-                  s_d[k + 1] -= f * s_du[k];
-                } else {
-                  const float f = s_d[k] / s_dl[k];
-                  s_d[k] = s_dl[k];
-                  s_dl[k] = f;
-                  const float t = s_du[k];
-                  s_du[k] = s_d[k + 1];
-                  s_d[k + 1] = t - f * s_d[k + 1];
-                  if (k + 2 < l) {
-                    s_du2[k] = s_du[k + 1];
-                    s_du[k + 1] = -f * s_du[k + 1];
-                  }
-                  s_piv[k] = 1;
-                }
-              }
-              // pivots below eps ||T|| are raised to it (a perturbation of
-              // T at rounding level) so the solves cannot overflow
-              for (int k = 0; k < l; ++k)
-                if (!(fabsf(s_d[k]) >= tiny)) s_d[k] = s_d[k] < 0.f ? -tiny : tiny;
-              for (int step = 0; step < 2; ++step) {
-                for (int k = 0; k + 1 < l; ++k) {
-                  if (s_piv[k]) {
-                    const float t = s_iv[k];
-                    s_iv[k] = s_iv[k + 1];
-                    s_iv[k + 1] = t - s_dl[k] * s_iv[k + 1];
-                  } else {
-                    s_iv[k + 1] -= s_dl[k] * s_iv[k];
-                  }
-                }
-                float mx = 0.f;
-                for (int k = l - 1; k >= 0; --k) {
-                  float v = s_iv[k];
-                  if (k + 1 < l) v -= s_du[k] * s_iv[k + 1];
-                  if (k + 2 < l) v -= s_du2[k] * s_iv[k + 2];
-                  v /= s_d[k];
-                  s_iv[k] = v;
-                  mx = fmaxf(mx, fabsf(v));
-                }
-                const float sc = mx > 0.f && mx <= FLT_MAX ? 1.f / mx : 0.f;
-                for (int k = 0; k < l; ++k) s_iv[k] = sc > 0.f ? s_iv[k] * sc : (k == a ? 1.f : 0.f);
-              }
-            }
-            __syncwarp();
-            float xa[4];
+  float x[4][4];  // vectors warp + 32 v, values lane + 32 u
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int r = lane + 32 * u;
-              xa[u] = r < l ? s_iv[r] : 0.f;
-            }
+  for (int v = 0; v < 4; ++v)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int g = warp + 32 * v, r = lane + 32 * u;
+      x[v][u] = g < l && r < l ? Z[r + (size_t)g * l] : 0.f;
+    }
+  int start = 0;
+  for (int i = 1; i <= l; ++i) {
+    if (i < l && lam[i] - lam[i - 1] <= ctol) continue;
+    for (int a = i - 1; a >= start && i - start > 1; --a) {
+      if (warp == (a & 31)) {
+        float q[4];
+        const int av = a >> 5;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float lo = av == 0 ? x[0][u] : x[1][u], hi = av == 2 ? x[2][u] : x[3][u];
+          q[u] = av < 2 ? lo : hi;
+        }
+        if (a < i - 1) {
+          float n2 = warp_sum(fmaf(q[0], q[0], fmaf(q[1], q[1], fmaf(q[2], q[2], q[3] * q[3]))));
+          if (n2 < 0.25f) {
+            inverse_iteration(s_inv, l, a, dd, ee, lam, q);
+            if (lane == 0) ++s_rep;
             for (int rep = 0; rep < 2; ++rep)
               for (int b = a + 1; b < i; ++b) {
                 float xb[4], dt = 0.f;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                  const int r = lane + 32 * u;
-                  xb[u] = r < l ? Xs[r * ldx + b] : 0.f;
-                  dt = fmaf(xa[u], xb[u], dt);
+                  xb[u] = Q[b * kMaxL + lane + 32 * u];
+                  dt = fmaf(q[u], xb[u], dt);
                 }
                 dt = warp_sum(dt);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) xa[u] = fmaf(-dt, xb[u], xa[u]);
+                for (int u = 0; u < 4; ++u) q[u] = fmaf(-dt, xb[u], q[u]);
               }
-            n2 = 0.f;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) n2 = fmaf(xa[u], xa[u], n2);
-            n2 = warp_sum(n2);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int r = lane + 32 * u;
-              if (r < l) Xs[r * ldx + a] = xa[u];
-            }
+            n2 = warp_sum(fmaf(q[0], q[0], fmaf(q[1], q[1], fmaf(q[2], q[2], q[3] * q[3]))));
           }
-          if (lane == 0) s_n2 = n2;
+          const float sc = n2 > 0.f ? rsqrtf(n2) : 0.f;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) q[u] *= sc;
         }
-        __syncthreads();
-        const float n2 = s_n2;
-        const float sc = n2 > 0.f ? rsqrtf(n2) : 0.f;
-        for (int r = tid; r < l; r += nt) Xs[r * ldx + a] *= sc;
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = lane + 32 * u;
+          Q[a * kMaxL + r] = q[u];
+          if (r < l) Z[r + (size_t)a * l] = q[u];
+        }
       }
-      start = i;
+      __syncthreads();
+      if (a > warp) {
+        float q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = Q[a * kMaxL + lane + 32 * u];
+        // vectors of this warp below a
+        switch ((a - warp + 31) >> 5) {
+          case 1: take_out<1>(x, q, warp, start); break;
+          case 2: take_out<2>(x, q, warp, start); break;
+          case 3: take_out<3>(x, q, warp, start); break;
+          default: take_out<4>(x, q, warp, start);
+        }
+      }
     }
-    // diagnostic word at byte 16 of the status block: replaced vectors
-    if (tid == 0) status[4] = (unsigned)nrep;
+    start = i;
   }
-
   __syncthreads();
-  for (int e = tid; e < l * l; e += nt) {
-    const int g = e / l, r = e - g * l;
-    Z[e] = Xs[r * ldx + g];
-  }
+  // diagnostic word at byte 16 of the status block: replaced vectors
+  if (tid == 0) status[4] = (unsigned)s_rep;
 }
 
 // Step 4: X = H_0 ... H_{l-2} Z for columns kBackCols blockIdx.x .. + 31,
