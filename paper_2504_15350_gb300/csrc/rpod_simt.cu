@@ -690,7 +690,12 @@ template <typename TP, typename TO>
 cudaError_t reduce_splits(cudaStream_t st, int64_t M, int64_t N, int nsplit, const TP* part,
                           TO* out, int64_t oi, int64_t oj) {
   const int64_t MN = M * N;
-  if (nsplit <= 32) {
+  // The flat kernel has one CTA per 1024 elements and takes the splits one after
+  // another: for an l x l Gram or the like (up to 128 x 128) the sliced one, with
+  // 32 elements a CTA, 9 -> 3 us at l = 30.  Not further: with the 64000 elements
+  // of a batch instance's T its many CTAs cost the other instances more (16 x
+  // 32768: 3090 -> 3215 us).
+  if (nsplit <= 32 && MN > 128 * 128) {
     const int vec = (sizeof(TP) == 4 && (MN & 3) == 0 && ((uintptr_t)part & 15) == 0) ? 1 : 0;
     k_reduce_flat<TP, TO><<<(unsigned)((MN + 1023) / 1024), 256, 0, st>>>(M, N, nsplit, part, out, oi,
                                                                           oj, vec);
