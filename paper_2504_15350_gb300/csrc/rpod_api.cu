@@ -337,9 +337,15 @@ struct Run {
     // Alg. 1: SVD of T via the eigenpairs of T T^T (FP64 Gram)
     double* GT = dbuf(P->off_g);
     const int ns = P->nsplit_t;
-    CK((gemm<W, W, W, double>(st, true, l, l, m, ns, Tt, m, Tt, m, dbuf(P->off_gpart), 1, l,
-                              (int64_t)l * l, status, false)));
-    CK((reduce_splits<double, double>(st, l, l, ns, dbuf(P->off_gpart), GT, 1, l)));
+    if constexpr (sizeof(W) == 4) {
+      float* const gp = (float*)dbuf(P->off_gpart);
+      CK((gram_t(st, m, l, Tt, m, ns, gp)));
+      CK((reduce_splits<float, double>(st, l, l, ns, gp, GT, 1, l)));
+    } else {
+      CK((gemm<W, W, W, double>(st, true, l, l, m, ns, Tt, m, Tt, m, dbuf(P->off_gpart), 1, l,
+                                (int64_t)l * l, status, false)));
+      CK((reduce_splits<double, double>(st, l, l, ns, dbuf(P->off_gpart), GT, 1, l)));
+    }
     double* Uhat = dbuf(P->off_uhat);
     if (sizeof(W) == 8) {
       // FP64 form: one-sided Jacobi sweeps on the transposed Cholesky factor

@@ -209,6 +209,9 @@ cudaError_t round_tf32(cudaStream_t st, int64_t rows, int64_t cols, const float*
 
 // FP64 partial Gram matrices part[z] = Y_z^T Y_z of nsplit row chunks of the
 // FP32 matrix Y (rows x l, l <= 128), products and chunk sums in FP32.
+// The same for the Gram of T^T: FP32 partials, only the upper triangle multiplied.
+cudaError_t gram_t(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
+                   float* part);
 cudaError_t gram_f32(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
                      double* part);
 

@@ -707,6 +707,7 @@ cudaError_t reduce_splits(cudaStream_t st, int64_t M, int64_t N, int nsplit, con
 }
 template cudaError_t reduce_splits<double, double>(cudaStream_t, int64_t, int64_t, int, const double*, double*, int64_t, int64_t);
 template cudaError_t reduce_splits<float, float>(cudaStream_t, int64_t, int64_t, int, const float*, float*, int64_t, int64_t);
+template cudaError_t reduce_splits<float, double>(cudaStream_t, int64_t, int64_t, int, const float*, double*, int64_t, int64_t);
 template cudaError_t reduce_splits<double, float>(cudaStream_t, int64_t, int64_t, int, const double*, float*, int64_t, int64_t);
 
 // ------------------------------------------------------------------------
@@ -2133,6 +2134,113 @@ k_gram_f32(int64_t rows, int l, const float* __restrict__ Y, int64_t ldy, int64_
       const int i = ty * 8 + a, j = tx * 8 + b;
       if (i < l && j < l) pz[i + j * l] = (double)acc[a][b];
     }
+}
+
+// Gram of T^T (rows = m snapshots, Alg. 1's small SVD) in FP32 partials of up to
+// 256 rows, any leading dimension.  Only the upper triangle is multiplied: its
+// 4 x 4 blocks (253 at l = 85, 528 at l = 128) go to consecutive threads, at most
+// two each, which add the rows of 32-row tiles in order, like the product on
+// 128 x 128 tiles that this replaces.  Where the chunks leave SMs idle, CTAs
+// (blockIdx.y) share the blocks, down to two warps each.
+// Bound: shared-memory reads (two of 16 bytes per 16 FMAs) and, for few
+// snapshots, the latency of a chunk.  Against that product, on 128 x 128 tiles
+// (120 us at 90225 x 85): basis of 8192 x 90225, BF16 (l = 85) 2969 -> 2903 us,
+// 4096 x 64000, FP32 (l = 60) 1364 -> 1337 us, 4096 x 500, FP16 (l = 30) 338 -> 330.
+constexpr int kGtThreads = 288;
+constexpr size_t kGtSmem = 528 * 17 * sizeof(float);
+__global__ void __launch_bounds__(kGtThreads)
+k_gram_t(int64_t rows, int l, const float* __restrict__ Y, int64_t ldy, int64_t chunk,
+         float* __restrict__ part) {
+  constexpr int BR = 32, LD = 132;
+  extern __shared__ __align__(16) float sgt[];  // two tiles [BR][LD], then the blocks' sums
+  static_assert(2 * BR * LD <= 528 * 17, "tiles fit");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nb = (l + 3) >> 2, T = nb * (nb + 1) / 2;
+  // this CTA's blocks [t0, t0 + tn); block (p, q), p <= q, is number
+  // q (q + 1) / 2 + p
+  const int per = (T + gridDim.y - 1) / gridDim.y, t0 = blockIdx.y * per, tn = min(per, T - t0);
+  int p[2], q[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int bq = 0, bp = min(t0 + tid + h * kGtThreads, T - 1);
+    while (bp > bq) bp -= ++bq;
+    p[h] = bp * 4;
+    q[h] = bq * 4;
+  }
+  const int64_t r0 = (int64_t)blockIdx.x * chunk;
+  const int64_t r1 = r0 + chunk < rows ? r0 + chunk : rows;
+  float acc[2][4][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[h][a][b] = 0.f;
+  // a lane's row of the tile, four columns at a time
+  float4 v[4];
+  auto load = [&](int64_t rb) {
+    const int64_t r = rb + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = 4 * (warp + 9 * u);
+      const float* y = Y + r + (int64_t)c * ldy;
+      const bool in = r < r1;
+      v[u].x = in && c < l ? y[0] : 0.f;
+      v[u].y = in && c + 1 < l ? y[ldy] : 0.f;
+      v[u].z = in && c + 2 < l ? y[2 * ldy] : 0.f;
+      v[u].w = in && c + 3 < l ? y[3 * ldy] : 0.f;
+    }
+  };
+  if (r0 < r1) load(r0);
+  float* tile = sgt;
+  for (int64_t rb = r0; rb < r1; rb += BR) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = 4 * (warp + 9 * u);
+      if (c < 4 * nb) *(float4*)&tile[lane * LD + c] = v[u];
+    }
+    __syncthreads();
+    if (rb + BR < r1) load(rb + BR);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (tid + h * kGtThreads < tn) {
+#pragma unroll 8
+        for (int rr = 0; rr < BR; ++rr) {
+          const float4 a4 = *(const float4*)&tile[rr * LD + p[h]], b4 = *(const float4*)&tile[rr * LD + q[h]];
+          const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[h][a][b] = fmaf(av[a], bv[b], acc[h][a][b]);
+        }
+      }
+    tile = tile == sgt ? sgt + BR * LD : sgt;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (tid + h * kGtThreads < tn) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) sgt[(tid + h * kGtThreads) * 17 + e] = acc[h][e >> 2][e & 3];
+    }
+  __syncthreads();
+  float* const pz = part + (int64_t)blockIdx.x * l * l;
+  for (int j = warp; j < l; j += kGtThreads / 32)
+    for (int i = lane; i < l; i += 32) {
+      const int lo = min(i, j), hi = max(i, j), qb = hi >> 2, t = qb * (qb + 1) / 2 + (lo >> 2) - t0;
+      if (t >= 0 && t < tn) pz[i + j * l] = sgt[t * 17 + (lo & 3) * 4 + (hi & 3)];
+    }
+}
+
+cudaError_t gram_t(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
+                   float* part) {
+  int64_t chunk = (rows + nsplit - 1) / nsplit;
+  chunk = (chunk + 15) / 16 * 16;
+  const int nb = (l + 3) / 4, T = nb * (nb + 1) / 2;
+  const int ny = std::max(1, std::min(152 / nsplit, (T + 63) / 64));
+  k_gram_t<<<dim3((unsigned)nsplit, (unsigned)ny), kGtThreads, kGtSmem, st>>>(rows, l, Y, ldy, chunk, part);
+  note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t gram_f32(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
