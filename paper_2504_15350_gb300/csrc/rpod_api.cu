@@ -304,33 +304,51 @@ struct Run {
     return RPOD_OK;
   }
 
+  // 16-bit forms: D = A B for A m x l (ld lda, a multiple of 4) and B l x N on
+  // the tensor cores with exactly split operands; UNSUPPORTED leaves the product
+  // to the caller.  B's parts go where the passes' 16-bit operands were (free
+  // after the last pass).  From 4096 rows on: below, the two launches take as
+  // long as the SIMT product (6 us at m = 500).  Fold and coefficients of
+  // 90225 x 85 took 74 and 43 us there; basis of 8192 x 90225: 2946 -> 2871 us,
+  // 262144 x 10000 unchanged.
+  int tall_product(int64_t M, int N, const W* A, int64_t lda, const W* B, W* D, int64_t di, int64_t dj) {
+    if constexpr (sizeof(W) == 4) {
+      if (is16(P->compute) && M >= 4096 && lda % 4 == 0 &&
+          P->off_qb + split_plane_bytes(P->l, N) <= P->off_wpart)
+        return split_gemm(st, false, M, N, P->l, A, lda, B, P->l, D, di, dj, ws + P->off_qb, nullptr, 0, 100,
+                          status, false);
+    }
+    return RPOD_ERR_UNSUPPORTED;
+  }
+
   // Fold a deferred last CholeskyQR factor into T: Tt (m x l) = Tt1 X,
-  // written to `out` (m x l).
-  int fold_t(const W* Tt1, W* out) {
+  // written to `out` (m x l, leading dimensions ld).
+  int fold_t(const W* Tt1, W* out, int64_t ld) {
     const int64_t m = P->m;
     const int l = P->l;
     // 16-bit forms: the two-part TF32 tensor-core product (about 2^-21
-    // relative error per entry, as the lift); else, or when Tt1 is not
-    // addressable by TMA, the SIMT product
+    // relative error per entry, as the lift) where m is a multiple of 4, else
+    // the split product; below its size, the SIMT product
     int rc = RPOD_ERR_UNSUPPORTED;
-    if (sizeof(W) == 4 && is16(P->compute))
-      rc = tc_apply(st, (const float*)Tt1, m, m, l, (const float*)buf(P->off_xw), l, (float*)out, m,
+    if (sizeof(W) == 4 && is16(P->compute) && m % 4 == 0)
+      rc = tc_apply(st, (const float*)Tt1, ld, m, l, (const float*)buf(P->off_xw), l, (float*)out, ld,
                     0, nullptr, 0, nullptr, 0, status, 0, true);
+    if (rc == RPOD_ERR_UNSUPPORTED) rc = tall_product(m, l, Tt1, ld, buf(P->off_xw), out, 1, ld);
     if (rc == RPOD_ERR_CUDA) return rc;
     if (rc != RPOD_OK) {
       if (P->compute == RPOD_F32)
-        CR(product(false, m, l, l, 1, Tt1, m, buf(P->off_xw), l, out, 1, m, false));
+        CR(product(false, m, l, l, 1, Tt1, ld, buf(P->off_xw), l, out, 1, ld, false));
       else
-        CK((gemm<W, W, W, W>(st, false, m, l, l, 1, Tt1, m, buf(P->off_xw), l, out, 1, m, 0, status,
+        CK((gemm<W, W, W, W>(st, false, m, l, l, 1, Tt1, ld, buf(P->off_xw), l, out, 1, ld, 0, status,
                              false)));
     }
     return RPOD_OK;
   }
 
-  // After T (as Tt, m x l): small SVD, lift, signs, coefficients.  With
+  // After T (as Tt, m x l, ld ldt): small SVD, lift, signs, coefficients.  With
   // `deferred` the basis is Q X (X from the deferred last CholeskyQR round)
   // and the lift uses X Uhat.
-  int finish(const W* Q, const W* Tt, W* U, int64_t ldu, double* sigma, W* C, int64_t ldc,
+  int finish(const W* Q, const W* Tt, int64_t ldt, W* U, int64_t ldu, double* sigma, W* C, int64_t ldc,
              bool deferred = false) {
     const int64_t n = P->n, m = P->m;
     const int l = P->l, k = P->k;
@@ -339,10 +357,10 @@ struct Run {
     const int ns = P->nsplit_t;
     if constexpr (sizeof(W) == 4) {
       float* const gp = (float*)dbuf(P->off_gpart);
-      CK((gram_t(st, m, l, Tt, m, ns, gp)));
+      CK((gram_t(st, m, l, Tt, ldt, ns, gp)));
       CK((reduce_splits<float, double>(st, l, l, ns, gp, GT, 1, l)));
     } else {
-      CK((gemm<W, W, W, double>(st, true, l, l, m, ns, Tt, m, Tt, m, dbuf(P->off_gpart), 1, l,
+      CK((gemm<W, W, W, double>(st, true, l, l, m, ns, Tt, ldt, Tt, ldt, dbuf(P->off_gpart), 1, l,
                                 (int64_t)l * l, status, false)));
       CK((reduce_splits<double, double>(st, l, l, ns, dbuf(P->off_gpart), GT, 1, l)));
     }
@@ -413,8 +431,10 @@ struct Run {
     // Sec. 4.3 coefficients C = U_k^T S = Uhat_k^T T (k x m), Uhat with the signs
     CK((convert_matrix<double, W>(st, l, k, Uhat, l, Uw, l)));
     if (P->compute == RPOD_F32)
-      return product(false, m, k, l, 1, Tt, m, Uw, l, C, ldc, 1, false);
-    CK((gemm<W, W, W, W>(st, false, m, k, l, 1, Tt, m, Uw, l, C, ldc, 1, 0, status, false)));
+      return product(false, m, k, l, 1, Tt, ldt, Uw, l, C, ldc, 1, false);
+    rc = tall_product(m, k, Tt, ldt, Uw, C, ldc, 1);
+    if (rc != RPOD_ERR_UNSUPPORTED) return rc;
+    CK((gemm<W, W, W, W>(st, false, m, k, l, 1, Tt, ldt, Uw, l, C, ldc, 1, 0, status, false)));
     return RPOD_OK;
   }
 
@@ -462,8 +482,8 @@ struct Run {
     CR(product(true, m, l, n, P->nsplit_z, S, lds, Q, n, Zq, 1, m, false));
     prof_end(P, st, pass_bytes, pass_flops);
     CR(exchange(Zq, m * l, sizeof(W) == 8 ? RPOD_F64 : RPOD_F32, RPOD_REDUCE_SUM));
-    CR(fold_t(Zq, Tt));
-    return finish(Q, Tt, U, ldu, sigma, C, ldc, true);
+    CR(fold_t(Zq, Tt, m));
+    return finish(Q, Tt, m, U, ldu, sigma, C, ldc, true);
   }
 
   // Tensor-core form (W = float): passes over a 16-bit S on tcgen05, the
@@ -482,6 +502,9 @@ struct Run {
     void* Qh = ws + P->off_qb;   // n_ld x 128, 16-bit
     void* Zh = ws + P->off_zb;   // m_ld x 128, 16-bit
     const int64_t nld = P->n_ld, mld = P->m_ld;
+    // Z and T with a 16-byte aligned leading dimension, so that their products
+    // take the tensor-core paths at any m
+    const int64_t m4 = round_up(m, 4);
     // Columns l..127 of the 16-bit operand buffers are never read: the tensor
     // maps span l columns and TMA fills the rest of each 128-wide box with 0.
     // the 16-bit S read by the passes
@@ -544,9 +567,6 @@ struct Run {
         prof_begin(P, st);
         CR(tc_wpass(st, dt, Qh, nld, n, l, Sh, ldh, m, wpart, P->nsplit_w, status, P->pass_stages));
         prof_end(P, st, pb16, pass_flops);
-        // Z with a 16-byte aligned leading dimension, so that its Gram
-        // takes the tensor-core path at any m
-        const int64_t m4 = round_up(m, 4);
         CK((reduce_splits<float, float>(st, m, l, P->nsplit_w, wpart, Z, 1, m4)));
         // the orthonormal Z goes straight to its 16-bit copy for the Y-pass
         // (the tensor-core apply; the SIMT product and a conversion when Z
@@ -598,12 +618,12 @@ struct Run {
       // accurate as FP32 ones (the 16-bit operands and the TF32 basis are
       // free by now and hold Q's parts)
       prof_begin(P, st);
-      CR(split_gemm(st, true, m, l, n, Sref, ldr, Q, n, Zq, 1, m, ws + P->off_qb,
+      CR(split_gemm(st, true, m, l, n, Sref, ldr, Q, n, Zq, 1, m4, ws + P->off_qb,
                     (float*)(ws + P->off_part), P->part_elems, P->split_pct, status, false));
       prof_end(P, st, 4.0 * ((double)n * m + (double)n * l + (double)m * l), pass_flops);
       CK(join());
-      CR(fold_t(Zq, Tt));
-      return finish(Q, Tt, U, ldu, sigma, C, ldc, true);
+      CR(fold_t(Zq, Tt, m4));
+      return finish(Q, Tt, m4, U, ldu, sigma, C, ldc, true);
     }
     if (refine) {
       if (!tf_ready) CK(round_tf32(st, n, l, Q, n, Atf, nld));
@@ -616,10 +636,10 @@ struct Run {
       CR(tc_wpass(st, dt, Qh, nld, n, l, Sh, ldh, m, wpart, P->nsplit_w, status, P->pass_stages));
       prof_end(P, st, pb16, pass_flops);
     }
-    CK((reduce_splits<float, float>(st, m, l, P->nsplit_w, wpart, Zq, 1, m)));
+    CK((reduce_splits<float, float>(st, m, l, P->nsplit_w, wpart, Zq, 1, m4)));
     CK(join());
-    CR(fold_t(Zq, Tt));
-    return finish(Q, Tt, U, ldu, sigma, C, ldc, true);
+    CR(fold_t(Zq, Tt, m4));
+    return finish(Q, Tt, m4, U, ldu, sigma, C, ldc, true);
   }
 
   int project(const W* U, int64_t ldu, int kc, const W* Sn, int64_t lds, int64_t mn, W* C,
@@ -744,7 +764,7 @@ static int plan_create_impl(rpod_plan** out, int64_t n, int64_t m, int32_t k, in
   P->off_q = take(w * n * L);
   P->off_z = take(w * round_up(m, 4) * L);
   P->off_zq = take(w * round_up(m, 4) * L);
-  P->off_tt = take(w * m * L);
+  P->off_tt = take(w * round_up(m, 4) * L);
   P->off_part = take(w * P->part_elems);
   P->off_gpart = take(8 * P->gpart_elems);
   P->off_g = take(8 * L * L);
