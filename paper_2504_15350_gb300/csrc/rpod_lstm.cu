@@ -15,11 +15,13 @@
 // kept when that word shifted right by 11 is at least ceil(p 2^53).  The
 // backward pass regenerates the same mask for the gradient it hands down.
 //
-// Kernels: the input projection of all T steps of a layer is one GEMM; each
-// recurrent step is one fused kernel (h_{t-1} W_h^T tile GEMM whose epilogue
-// applies the gate activations and the c/h update); BPTT runs one fused
-// pointwise kernel (gate gradients, dc) and one GEMM (dz W_h) per step, then
-// three GEMMs over all steps for dW_x, dW_h and the input gradient.
+// With BF16 weights the passes run in rpod_lstm_mma.cu (one launch per layer +
+// time anti-diagonal).  With FP32 weights the kernels are here: the input
+// projection of all T steps of a layer is one GEMM; each recurrent step is one
+// fused kernel (h_{t-1} W_h^T tile GEMM whose epilogue applies the gate
+// activations and the c/h update); BPTT runs one fused pointwise kernel (gate
+// gradients, dc) and one GEMM (dz W_h) per step, then three GEMMs over all steps
+// for dW_x, dW_h and the input gradient.
 #include <math.h>
 
 #include <stdio.h>

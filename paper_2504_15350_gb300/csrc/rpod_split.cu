@@ -36,10 +36,10 @@
 //
 // Bound: 6 bf16 products per value, so at N = 128 the tensor cores need as
 // long for a tile as HBM (1536 clocks per 32 KB at 4096 FMA a clock and SM);
-// at N = 64 HBM alone.  Measured (products of 1.05 GB, with the planes and the
-// sum of the partials): S^T Q at 65536 x 4000, l = 120, 357 us and S Z 376 us
-// (1640 and 1600 us on the FP32 pipes); at 4096 x 64000, l = 60, 364 and 326 us
-// (1400 and 6600 us, the latter on 32 CTAs).
+// at N = 64 HBM alone.  Measured (kernel alone, products of 1.05 GB, 155 us of
+// HBM): S^T Q at 65536 x 4000, l = 120, 245 us and S Z 267 us (1640 and 1600 us on
+// the FP32 pipes); at 4096 x 64000, l = 60, 205 and 170 us (1400 and 6600 us, the
+// latter on 32 CTAs).
 #include <algorithm>
 #include <mutex>
 
