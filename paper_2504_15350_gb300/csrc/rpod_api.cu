@@ -188,7 +188,7 @@ struct Run {
   // pipes.
   int gram(const W* A, int64_t rows, int64_t lda, double* G, int nsplit, bool fast) {
     const int l = P->l;
-    if (sizeof(W) == 4) {
+    if constexpr (sizeof(W) == 4) {
       // the exact kernel holds one CTA per SM: one wave of partials
       const int ns = fast ? nsplit : std::min(nsplit, tc_sm_count());
       float* fpart = (float*)dbuf(P->off_gpart);

@@ -564,7 +564,6 @@ cudaError_t gemm(cudaStream_t st, bool akc, int64_t M, int64_t N, int64_t K, int
                                                unsigned*, bool);
 INST_GEMM(double, double, double, double)
 INST_GEMM(float, float, float, float)
-INST_GEMM(float, float, float, double)
 INST_GEMM(float, double, float, float)
 INST_GEMM(double, double, double, float)
 #undef INST_GEMM
