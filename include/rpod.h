@@ -352,7 +352,9 @@ void rpod_batch_destroy(rpod_batch* batch);
  * The caller's workspace (rpod_lstm_workspace_bytes) holds the parameters,
  * the Adam moments and all activations: keep it for the life of the model.
  * Inputs X are row-major (batch, window, in_dim) FP32 device arrays, targets
- * and outputs row-major (batch, out_dim). */
+ * and outputs row-major (batch, out_dim).  An infinite window entry saturates
+ * the gates that it reaches, as in FP32 arithmetic; where it meets a weight or a
+ * gradient of zero the product is NaN. */
 typedef struct rpod_lstm rpod_lstm;
 
 /* rpod_lstm_create flags */

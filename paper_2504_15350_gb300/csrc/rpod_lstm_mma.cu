@@ -30,6 +30,8 @@
 // 4045 us with FP32 products and about 100 launches; a training step at 3 x 50,
 // batch 16: 157 us (1570 us).
 #include <cooperative_groups.h>
+#include <float.h>
+#include <math.h>
 
 #include <algorithm>
 #include <utility>
@@ -43,11 +45,15 @@ constexpr int kLd = 72;  // bf16 per staged row: 64 values and 16 bytes
 
 __device__ __forceinline__ float sigm_m(float x) { return 1.f / (1.f + __expf(-x)); }
 
-// a = a1 + a2 + a3 for two values, packed as bf16 pairs (low half a)
+// a = a1 + a2 + a3 for two values, packed as bf16 pairs (low half a).  An
+// infinity is (a, 0, 0): the difference to its first part would be NaN, and
+// with it every sum that the infinity alone leaves infinite (a window with an
+// infinite entry saturates its gates, as with FP32 products).
 __device__ __forceinline__ void parts3(float a, float b, uint32_t (&p)[3]) {
   const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
   p[0] = __byte_perm(ua, ub, 0x7632);
-  const float ra = a - __uint_as_float(ua & 0xffff0000u), rb = b - __uint_as_float(ub & 0xffff0000u);
+  const float ra = fabsf(a) == INFINITY ? 0.f : a - __uint_as_float(ua & 0xffff0000u);
+  const float rb = fabsf(b) == INFINITY ? 0.f : b - __uint_as_float(ub & 0xffff0000u);
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[1]) : "f"(rb), "f"(ra));
   const float qa = ra - __uint_as_float(p[1] << 16), qb = rb - __uint_as_float(p[1] & 0xffff0000u);
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[2]) : "f"(qb), "f"(qa));
@@ -590,7 +596,8 @@ __global__ void __cluster_dims__(1, kSumSplit, 1) __launch_bounds__(1024) k_lstm
     }
   }
 #pragma unroll
-  for (int j = 0; j < 2; ++j) part[ty][2 * lane + j] = (double)s[j] + (double)err[j];
+  for (int j = 0; j < 2; ++j)  // an infinite sum has no error term (TwoSum's is NaN)
+    part[ty][2 * lane + j] = (double)s[j] + (fabsf(s[j]) <= FLT_MAX ? (double)err[j] : 0.0);
   __syncthreads();
   if (threadIdx.x < 64) {
     double t = 0.0;
