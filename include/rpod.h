@@ -79,7 +79,11 @@ typedef enum {
 /* Warning bits returned through rpod_status_sync()'s flags_out. */
 enum {
   RPOD_WARN_RANK_DEFICIENT = 1u  /* a Gram matrix had numerically dependent
-                                    columns; the matching basis columns are 0 */
+                                    columns: less than 1e-13 of a column's squared
+                                    norm (FP32 and 16-bit forms: 1e-5 in rounds
+                                    after the first) is left after the columns
+                                    before it.  See rpod_basis for what the
+                                    matching basis columns hold */
 };
 
 /* Plan flags. */
@@ -154,8 +158,12 @@ int rpod_workspace_bytes(const rpod_plan* plan, size_t* bytes);
  *   C:         k x m modal coefficients U_k^T S, ldc >= k; double for F64,
  *              float otherwise.
  * Column signs: each column of U has its largest-magnitude entry positive;
- * C's rows follow.  Columns of U that belong to numerically rank-deficient
- * directions are zero (flagged by RPOD_WARN_RANK_DEFICIENT). */
+ * C's rows follow.  Numerically rank-deficient directions are flagged by
+ * RPOD_WARN_RANK_DEFICIENT and their columns of U are zero, but in the FP32
+ * form: there they come after the resolved ones with singular values at
+ * rounding level (below 1e-5 sigma_1) and hold rounding noise, orthogonal to
+ * the resolved columns; many of them (an l far above the rank) need not have
+ * norm 1 nor be orthogonal to one another. */
 int rpod_basis(rpod_plan* plan, const void* S, int64_t lds, int32_t s_dtype,
                const float* S_refine, int64_t ldr,
                void* U, int64_t ldu, double* sigma, void* C, int64_t ldc,

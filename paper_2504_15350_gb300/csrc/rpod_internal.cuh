@@ -131,7 +131,8 @@ cudaError_t sketch(cudaStream_t st, uint64_t seed, uint64_t stream_id, int64_t m
 // ST_RANK_DEF, without dropping, for columns of squared norm below 1e-16
 // (rounds after a shifted one, whose basis is near orthonormal).
 // FP32 working type: shift_coef raises the diagonal of the gated FP64
-// factorization's Gram by that share of itself.
+// factorization's Gram by that share of itself; columns whose pivot without
+// the raise is below 1e-13 of the diagonal raise ST_RANK_DEF and are kept.
 // gate_second (FP32 working type, round 1): the second round takes the same
 // gated FP64 factorization when its FP32 pivots show kappa(Q1)^2 > 2.
 template <typename TW>

@@ -1426,7 +1426,7 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
   // other threads finish the step, so a column costs one barrier.
   const int cb = tid & 127, rg = tid >> 7, ng = nt >> 7;
   auto pivot = [&](int j, double d) {
-    const bool keep = (d0[j] > 1e-300) && (d0[j] > 1e-30 * gmax) && (d > 1e-13 * d0[j]);
+    const bool keep = (d0[j] > 1e-300) && (d0[j] > 1e-30 * gmax) && (d > tol * d0[j]);
     const double ri = keep ? rsqrt(d) : 0.0;
     s_keep[j] = keep ? 1 : 0;
     s_ri[j] = ri;
@@ -1481,13 +1481,28 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
     if (Xout) Xout[e] = (double)v;
     Xw[i + (int64_t)j * ldxw] = (TW)v;
   }
+  // The pivots above are those of the raised matrix, never below reg d0.  The
+  // pivot that the matrix itself has -- the squared norm left of the column
+  // after the ones before it -- is what is left of the column in Q1 = Y X,
+  // 1 - reg sum_i d0_i X_ij^2, times the raised one; a column that it shows to
+  // be dependent keeps its place (the raise completes it to a direction at
+  // rounding level) and is reported.
+  if (reg > 0.0 && tid < l && s_keep[tid]) {
+    const int j = tid;
+    double raise = 0.0;
+    for (int i = 0; i <= j; ++i) {
+      const double x = Xf[(size_t)i * ldx + j];
+      raise = fma(d0[i] * x, x, raise);
+    }
+    const double r = 1.0 / rf[j];
+    if ((1.0 - reg * raise) * r * r <= tol * d0[j]) atomicOr(status, ST_RANK_DEF);
+  }
   if (tid == 0) {
     int ndropped = 0;
     for (int j = 0; j < l; ++j) ndropped += s_keep[j] ? 0 : 1;
     *gate = 0;
     if (ndropped > 0) atomicOr(status, ndropped == l ? (ST_RANK_DEF | ST_BREAKDOWN) : ST_RANK_DEF);
   }
-  (void)tol;
 }
 template cudaError_t cholesky<double>(cudaStream_t, int, const void*, double, int, double*, double*, int, unsigned*, const float*, int64_t, double*, int, int64_t, double, bool, bool);
 template cudaError_t cholesky<float>(cudaStream_t, int, const void*, double, int, double*, float*, int, unsigned*, const float*, int64_t, double*, int, int64_t, double, bool, bool);
