@@ -221,8 +221,9 @@ cudaError_t gram_f32(cudaStream_t st, int64_t rows, int l, const float* Y, int64
 // B x H states, count/abort_word/status: zeroed words (barrier arrivals, the
 // abort word, the status word).  rollout_units: hidden units per CTA;
 // rollout_smem_bytes: dynamic shared memory of one CTA (the caller checks it
-// against the device limit).  grid_sync_selftest: the barrier with one CTA
+// against kRollSmemMax).  grid_sync_selftest: the barrier with one CTA
 // that never arrives, limited to `seconds`; returns the status word left.
+constexpr size_t kRollSmemMax = (size_t)200 * 1024;
 int rollout_units(int H, int sms);
 size_t rollout_smem_bytes(int I, int H, int L, int O, int B, int U);
 cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,

@@ -761,7 +761,7 @@ int rpod_lstm_gather(const rpod_lstm* N, const float* series, const float* mu, i
 static bool rollout_fits(const rpod_lstm* N, int B, int sms) {
   if (N->L > 4) return false;
   const int U = rollout_units(N->H, sms);
-  return rollout_smem_bytes(N->I, N->H, N->L, N->O, B, U) <= (size_t)200 * 1024;
+  return rollout_smem_bytes(N->I, N->H, N->L, N->O, B, U) <= kRollSmemMax;
 }
 
 int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_cols, int32_t steps,

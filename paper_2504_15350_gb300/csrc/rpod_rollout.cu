@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(512, 1) k_rollout(RollArgs a) {
 // at 2 x 256, window 10, 8 samples, 500 steps: 4.1 ms; the kernel with
 // T + L - 1 grid barriers per prediction above takes 68.4 ms.
 constexpr int kPipeThreads = 384;
+constexpr size_t kPipeSmemMax = (size_t)226 * 1024;
 
 struct PipeArgs {
   int I, H, L, O, T, d, U, CS, steps;
@@ -688,15 +689,11 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
   const size_t smem = rollout_smem_bytes(I, H, L, O, B, a.U);
   const dim3 grid((unsigned)(H / a.U)), block(512);
   void* args[] = {&a};
-  cudaError_t e;
-  if (bf16_weights) {
-    e = cudaFuncSetAttribute(k_rollout<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaLaunchCooperativeKernel((void*)k_rollout<__nv_bfloat16>, grid, block, args, smem, st);
-  } else {
-    e = cudaFuncSetAttribute(k_rollout<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel((void*)k_rollout<float>, grid, block, args, smem, st);
-  }
+  const void* fn = bf16_weights ? (const void*)k_rollout<__nv_bfloat16> : (const void*)k_rollout<float>;
+  if (smem > kRollSmemMax) return cudaErrorCooperativeLaunchTooLarge;
+  // the kernel's largest size, not this network's: see pipe_launch
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRollSmemMax);
+  if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, grid, block, args, smem, st);
   note_launch();
   return e;
 }
@@ -704,12 +701,14 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
 namespace {
 
 // One cluster per sample: the launch, or with `active` only how many clusters
-// run at once (nothing enqueued).
+// run at once (nothing enqueued).  The attributes are the kernel's on this
+// device, for every thread: always set to the same values, so that no thread
+// lowers them between another's call and its launch.
 template <typename TW, int NP>
 cudaError_t pipe_launch(cudaStream_t st, const PipeArgs& a, int B, size_t smem, int* active) {
   auto fn = k_rollout_pipe<TW, NP>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && a.CS > 8)
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmemMax);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -785,7 +784,7 @@ cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, 
   double best = 0.0;
   for (int CS : {16, 12, 8, 4, 2, 1}) {
     const size_t smem = shape(CS);
-    if (smem > (size_t)226 * 1024 || (CS > 1 && H < 2 * CS)) continue;
+    if (smem > kPipeSmemMax || (CS > 1 && H < 2 * CS)) continue;
     const int active = bf16_weights ? pipe_active<__nv_bfloat16>(a, np, smem)
                                     : pipe_active<float>(a, np, smem);
     if (active < 1) continue;
