@@ -402,14 +402,18 @@ int rpod_lstm_gather(const rpod_lstm* net, const float* series, const float* mu,
                      float* X, float* Y, void* stream);
 /* Autoregressive prediction (the online stage): from the window (B, window,
  * in_dim), predict, append [mu of the newest row, prediction] as the newest
- * row, drop the oldest, `steps` times; out (B, steps, out_dim).  Runs as one
- * persistent cooperative kernel when the network fits (at most 4 layers; the
- * gate rows of a CTA's hidden units plus the staged inputs of B windows
- * within 200 KB of shared memory): the weights stay in shared memory for all
- * steps, and a grid barrier separates the anti-diagonal phases of the
- * layer x time cells; every barrier wait is limited to 2 s, after which the
- * kernel records RPOD_ERR_TIMEOUT (read by rpod_lstm_status_sync) and
- * returns.  Otherwise one series of kernels per step. */
+ * row, drop the oldest, `steps` times; out (B, steps, out_dim).  Runs in one of
+ * three ways, the one with the least estimated time:
+ *   - one kernel with a thread-block cluster per sample, in which all windows
+ *     that share a row advance together (at most 4 layers, a window of at most
+ *     16, the cluster's share of the weights within shared memory);
+ *   - one persistent cooperative kernel (at most 4 layers; the gate rows of a
+ *     CTA's hidden units plus the staged inputs of B windows within 200 KB of
+ *     shared memory): the weights stay in shared memory for all steps, and a
+ *     grid barrier separates the anti-diagonal phases of the layer x time cells;
+ *   - the kernels of rpod_lstm_forward for every step (many windows, few steps).
+ * In the first two every wait is limited to 2 s, after which the kernel records
+ * RPOD_ERR_TIMEOUT (read by rpod_lstm_status_sync) and returns. */
 int rpod_lstm_rollout(rpod_lstm* net, const float* window, int32_t B, int32_t mu_cols,
                       int32_t steps, float* out, void* workspace, size_t workspace_bytes,
                       void* stream);
@@ -459,7 +463,7 @@ int rpod_lstm_dims(const rpod_lstm* net, int32_t* dims);
 int rpod_lstm_set_dropout(rpod_lstm* net, double p, uint64_t seed);
 int rpod_lstm_last_launch_count(const rpod_lstm* net);
 /* Synchronises `stream`, reads and clears the network's device status word
- * (set by a persistent rollout whose barrier wait ran out): RPOD_ERR_TIMEOUT
+ * (set by a rollout kernel whose wait ran out): RPOD_ERR_TIMEOUT
  * or RPOD_OK.  Errors: RPOD_ERR_INVALID_ARG for NULL arguments. */
 int rpod_lstm_status_sync(const rpod_lstm* net, void* workspace, void* stream);
 

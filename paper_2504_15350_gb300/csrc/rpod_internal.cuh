@@ -233,11 +233,12 @@ cudaError_t rollout_persistent(cudaStream_t st, bool bf16_weights, int I, int H,
                                int* abort_word, unsigned* status, int sms);
 // The pipelined form over a thread-block cluster per sample (window: B x T x I
 // as given, not modified): cudaErrorInvalidConfiguration, with nothing
-// enqueued, when the network does not fit (L > 4, T > 16, shared memory).
+// enqueued, when the network does not fit (L > 4, T > 16, shared memory) or the
+// call would take longer than limit_us by its estimate.
 cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,
                               int B, int d, int steps, const float* theta, const void* wbf,
                               const int64_t (*off_w)[3], int64_t off_wy, int64_t off_by,
-                              const float* window, float* out, unsigned* status);
+                              const float* window, float* out, unsigned* status, double limit_us);
 cudaError_t grid_sync_selftest(cudaStream_t st, double seconds, unsigned* status_out);
 
 // Sets every kernel attribute the library needs (dynamic shared memory

@@ -764,6 +764,28 @@ static bool rollout_fits(const rpod_lstm* N, int B, int sms) {
   return rollout_smem_bytes(N->I, N->H, N->L, N->O, B, U) <= kRollSmemMax;
 }
 
+// Estimated us of a rollout in a prediction's own kernels, and in the persistent
+// kernel, measured as rollout_pipelined's (within a fifth; odd sizes of the BF16
+// kernels half as much again).  With them the pipelined kernel, whose waves
+// each load the weights and run `window` rows before the first prediction, is
+// left for the per-step kernels where many windows take few steps: 512 windows
+// of 2 x 256 take 255 us for one step and 2.26 ms for ten instead of 7.7 and
+// 12.1 ms (0.89 and 8.6 ms in FP32 kernels); 64 windows 169 us for one and 14.0
+// ms in the pipelined kernel for 200 (28.3 ms per step).
+static double rollout_steps_us(const rpod_lstm* N, int B, int steps) {
+  const double H = N->H, phases = N->L + N->T - 1;
+  if (N->wfp32) return 25.0 + steps * (N->L * N->T * (7.0 + 0.1 * H) * (1.0 + B / 3000.0));
+  const int chunks = (std::max(N->I, N->L > 1 ? N->H : 0) + 63) / 64 + (N->H + 63) / 64;
+  double us = 0.6 * chunks;  // of a phase: 16-row tiles up to 32 rows, then 64-row ones
+  if (B > 32) us = 1.3 * chunks * std::max(1.0, (B + 63) / 64 * ((N->H + 15) / 16) * std::min(N->L, N->T) / 152.0);
+  const double odd = ((N->H | N->I) & 1) ? 1.5 : 1.0;
+  return 25.0 + steps * (8.0 + odd * phases * (2.0 + us));
+}
+static double rollout_persistent_us(const rpod_lstm* N, int B, int steps, int sms) {
+  const double phases = N->L + N->T - 1;
+  return 25.0 + steps * phases * (3.6 + 1.2 * N->L + 1e-3 * rollout_units(N->H, sms) * N->H * B);
+}
+
 int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_cols, int32_t steps,
                       float* out, void* ws, size_t bytes, void* stream) {
   rpod::NvtxRange nv("rpod_lstm_rollout");
@@ -774,13 +796,19 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
   cudaStream_t st = (cudaStream_t)stream;
   Net net{N, (char*)ws, st};
   g_launches = 0;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return RPOD_ERR_CUDA;
   unsigned* sync = (unsigned*)((char*)ws + N->o_sync);
   LK(cudaMemsetAsync(sync, 0, 16, st));  // barrier arrivals, abort word, status word
+  const double step_us = rollout_steps_us(N, B, steps);
+  const bool persistent = rollout_fits(N, B, sms) && rollout_persistent_us(N, B, steps, sms) < step_us;
   {
     const cudaError_t e = rollout_pipelined(
         st, !N->wfp32, N->I, N->H, N->L, N->O, N->T, B, mu_cols, steps, net.f(N->o_theta),
         N->wfp32 ? (const void*)net.f(N->o_theta) : (const void*)net.wbf(), N->off_w, N->off_wy,
-        N->off_by, window, out, sync + 2);
+        N->off_by, window, out, sync + 2, persistent ? rollout_persistent_us(N, B, steps, sms) : step_us);
     if (e == cudaSuccess) {
       N->last_launches = g_launches;
       return RPOD_OK;
@@ -791,11 +819,7 @@ int rpod_lstm_rollout(rpod_lstm* N, const float* window, int32_t B, int32_t mu_c
   float* nxt = net.f(N->o_xtm2);
   k_to_time_major<<<blocks_for((int64_t)B * N->T * N->I), 256, 0, st>>>(B, N->T, N->I, window, cur);
   LL();
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return RPOD_ERR_CUDA;
-  if (rollout_fits(N, B, sms)) {
+  if (persistent) {
     // one cooperative launch for all steps (the window in o_xtm is its ring)
     const cudaError_t e = rollout_persistent(
         st, !N->wfp32, N->I, N->H, N->L, N->O, N->T, B, mu_cols, steps, net.f(N->o_theta),

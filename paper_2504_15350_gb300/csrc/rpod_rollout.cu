@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "rpod_internal.cuh"
 
@@ -738,13 +739,31 @@ cudaError_t pipe_np(cudaStream_t st, const PipeArgs& a, int B, int np, size_t sm
   }
 }
 
+// How many clusters of a shape run at once on the current device, kept for the
+// last 64 shapes asked for: a query takes about 2 us, the six of a call as long
+// as a whole prediction of a small network.
 template <typename TW>
 int pipe_active(const PipeArgs& a, int np, size_t smem) {
+  struct Entry {
+    int dev, np, cs, active;
+    size_t smem;
+  };
+  static std::mutex lock;
+  static Entry known[64];
+  static unsigned count = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> hold(lock);
+  for (unsigned i = 0; i < count && i < 64; ++i) {
+    const Entry& k = known[i];
+    if (k.dev == dev && k.np == np && k.cs == a.CS && k.smem == smem) return k.active;
+  }
   int n = 0;
   if (pipe_np<TW>(nullptr, a, 1, np, smem, &n) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
+  known[count++ % 64] = {dev, np, a.CS, n, smem};
   return n;
 }
 
@@ -753,7 +772,7 @@ int pipe_active(const PipeArgs& a, int np, size_t smem) {
 cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, int L, int O, int T,
                               int B, int d, int steps, const float* theta, const void* wbf,
                               const int64_t (*off_w)[3], int64_t off_wy, int64_t off_by,
-                              const float* window, float* out, unsigned* status) {
+                              const float* window, float* out, unsigned* status, double limit_us) {
   if (L > 4 || T > 16) return cudaErrorInvalidConfiguration;
   const int np = T <= 4 ? 2 : (T <= 8 ? 4 : (T <= 10 ? 5 : (T <= 12 ? 6 : 8)));
   const size_t wsz = bf16_weights ? 2 : 4;
@@ -780,7 +799,21 @@ cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, 
     a.threads = a.SL * 2 * a.U;
     return a.SL < 1 ? (size_t)-1 : pipe_smem_bytes(I, H, L, O, a.U, CS, 2 * np, a.SL, wsz);
   };
-  int pick = 0;
+  // Whole call in us, measured at seven networks (20 to 256 units, windows of 4
+  // to 16), 1 to 4096 samples, 1 to 200 steps, BF16 and FP32 weights: each wave
+  // loads the weights (0.56 us per 1000 of a CTA) and runs T + steps rows of L
+  // phases and the products; within a fifth of the measured times.
+  auto call_us = [&](int waves) {
+    double weights = 0.0;
+    for (int l = 0; l < L; ++l) weights += 4.0 * a.U * ((l == 0 ? I : H) + H);
+    const double products = 4.0 * a.U * 2 * np * (2.0 * L - 1.0) * H / 128.0;  // clocks
+    const double row = 0.6 + 1.45 * L + 1.9 * products / 2030.0 + 0.2 * L * std::max(0, 2 * np - 12);
+    return 25.0 + waves * (4.0 + 0.56e-3 * weights + (T + steps) * row);
+  };
+  // no cluster size can do better than all samples at once on the fewest units
+  shape(16);
+  if (call_us(1) > limit_us) return cudaErrorInvalidConfiguration;
+  int pick = 0, waves = 1;
   double best = 0.0;
   for (int CS : {16, 12, 8, 4, 2, 1}) {
     const size_t smem = shape(CS);
@@ -789,14 +822,17 @@ cudaError_t rollout_pipelined(cudaStream_t st, bool bf16_weights, int I, int H, 
                                     : pipe_active<float>(a, np, smem);
     if (active < 1) continue;
     const double products = 4.0 * a.U * 2 * np * (2.0 * L - 1.0) * H / 128.0;
-    const double cost = (double)((B + active - 1) / active) * (1.5 * products + 1500.0 * L);
+    const int w = (B + active - 1) / active;
+    const double cost = (double)w * (1.5 * products + 1500.0 * L);
     if (!pick || cost < best) {
       pick = CS;
       best = cost;
+      waves = w;
     }
   }
   if (!pick) return cudaErrorInvalidConfiguration;
   const size_t smem = shape(pick);
+  if (call_us(waves) > limit_us) return cudaErrorInvalidConfiguration;
   const cudaError_t e = bf16_weights ? pipe_np<__nv_bfloat16>(st, a, B, np, smem, nullptr)
                                      : pipe_np<float>(st, a, B, np, smem, nullptr);
   if (e == cudaSuccess) note_launch();

@@ -846,6 +846,6 @@ class LSTM:
         return rpod_lstm_last_launch_count(self.handle)
 
     def status(self):
-        """Device status of the last persistent rollout (RPOD_OK or
+        """Device status of the last rollout (RPOD_OK or
         RPOD_ERR_TIMEOUT); synchronises the stream."""
         return rpod_lstm_status_sync(self.handle, self.ws_ptr, self._stream())
