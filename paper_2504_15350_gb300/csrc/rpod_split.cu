@@ -32,7 +32,7 @@
 // skinny side's re-reads load the shared memory, which a 128 x 128 MMA with
 // both operands there would saturate.  An A that TMA cannot address (base or
 // leading dimension not a multiple of 16 bytes) is staged by 4-byte cp.async
-// from warps 19-20 instead.
+// from warps 0, 19 and 20 instead.
 //
 // Bound: 6 bf16 products per value, so at N = 128 the tensor cores need as
 // long for a tile as HBM (1536 clocks per 32 KB at 4096 FMA a clock and SM);
@@ -135,7 +135,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < RS; ++s) {
-      mbar_init(&rfull[s], TMA ? 1 : 64);
+      mbar_init(&rfull[s], TMA ? 1 : 96);
       mbar_init(&rempty[s], 4);
     }
     for (int s = 0; s < BS; ++s) {
@@ -330,8 +330,15 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           if (half * NH + c < g.N) o[c * g.dj] = acc[c];
       }
     }
-  } else if (!TMA && warp >= 19) {
-    const int t = threadIdx.x - 19 * 32;
+  } else if (!TMA && (warp == 0 || warp >= 19)) {
+    // Three warps, each a line of the tile (!KC: 128 rows of one k; KC: 64 k of
+    // one row) in turn.  A whole tile takes the loop without conditions, whose
+    // 32 copies in flight per lane hide the loads' latency: with a condition and
+    // an index computation per copy, about five were in flight, and a k-block took
+    // 8.7 us (!KC) or 4.2 us; now 1.1 us.  S^T Q and S Z of 65537 x 4000 by
+    // 128: 428 and 390 us (FP32 FMAs 1950 us).
+    const int w3 = warp == 0 ? 0 : warp - 18;
+    constexpr int LN = KC ? 128 : 64, PER = KC ? 2 : 4;  // lines, 32-value pieces of one
     int it = 0;
     bool go = true;
     for (int64_t w = blockIdx.x; w < g.items && go; w += gridDim.x) {
@@ -343,26 +350,33 @@ k_split_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
           go = false;
           break;
         }
+        const int64_t k0 = (int64_t)kb * 64, l0 = KC ? i0 : k0, c0 = KC ? k0 : i0;
+        const int nl = (int)min((int64_t)LN, (KC ? g.M : g.K) - l0);  // lines inside A
+        const int nc = (int)min((int64_t)(32 * PER), (KC ? g.K : g.M) - c0) - lane;  // a line's values from here on
         const uint32_t dst = su32(smem + s * L::RAW);
-        const int64_t k0 = (int64_t)kb * 64;
+        const float* src = g.A + c0 + lane + (l0 + w3) * g.lda;
+        auto at = [&](int ln, int h) {  // byte offset in the slot
+          return KC ? (uint32_t)(h * 16384 + ln * 128 + (((lane >> 2) ^ (ln & 7)) << 4) + (lane & 3) * 4)
+                    : (uint32_t)(ln * 512 + (32 * h + lane) * 4);
+        };
+        if (nl == LN && nc + lane == 32 * PER) {
 #pragma unroll 8
-        for (int e = t; e < 128 * 64; e += 64) {
-          int i, k;
-          uint32_t off;
-          if (KC) {
-            k = e & 63;
-            i = e >> 6;
-            off = (uint32_t)((k >> 5) * 16384 + i * 128 + ((((k & 31) >> 2) ^ (i & 7)) << 4) + (k & 3) * 4);
-          } else {
-            i = e & 127;
-            k = e >> 7;
-            off = (uint32_t)(k * 512 + i * 4);
+          for (int ln = w3; ln < LN; ln += 3, src += 3 * g.lda) {
+#pragma unroll
+            for (int h = 0; h < PER; ++h)
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + at(ln, h)), "l"(src + 32 * h)
+                           : "memory");
           }
-          const bool in = i0 + i < g.M && k0 + k < g.K;
-          const float* src = in ? g.A + (KC ? (k0 + k) + (i0 + i) * g.lda : (i0 + i) + (k0 + k) * g.lda) : g.A;
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + off), "l"(src),
-                       "r"(in ? 4 : 0)
-                       : "memory");
+        } else {
+          for (int ln = w3; ln < LN; ln += 3, src += 3 * g.lda) {
+#pragma unroll
+            for (int h = 0; h < PER; ++h) {
+              const bool in = ln < nl && 32 * h < nc;
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + at(ln, h)),
+                           "l"(in ? src + 32 * h : g.A), "r"(in ? 4 : 0)
+                           : "memory");
+            }
+          }
         }
         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(su32(&rfull[s])) : "memory");
       }
