@@ -685,20 +685,51 @@ k_reduce_flat(int64_t M, int64_t N, int nsplit, const TP* __restrict__ part, TO*
   }
 }
 
+// Up to 8 splits of an l x l output: one thread per element, all its partials in
+// flight, no shared memory.  k_reduce takes as long alone, but starts eight
+// threads per element, and in a batch those of one instance wait for slots
+// beside the other instances' kernels: 64 instances of 2000 x (300 to 900), BF16,
+// 1033 -> 972 us at l = 30 and 2685 -> 2412 us at l = 100.
+template <typename TP, typename TO>
+__global__ void __launch_bounds__(128)
+k_reduce_few(int64_t M, int64_t N, int nsplit, const TP* __restrict__ part, TO* __restrict__ out,
+             int64_t oi, int64_t oj) {
+  const int64_t MN = M * N, idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (idx >= MN) return;
+  TP v[8];
+#pragma unroll
+  for (int z = 0; z < 8; ++z) v[z] = z < nsplit ? part[(int64_t)z * MN + idx] : TP(0);
+  double t;
+  if constexpr (sizeof(TP) == 8) {
+    t = v[0];
+#pragma unroll
+    for (int z = 1; z < 8; ++z)
+      if (z < nsplit) t += v[z];
+  } else {
+    float s = v[0], c = 0.f;
+#pragma unroll
+    for (int z = 1; z < 8; ++z) two_sum_acc(s, c, v[z]);
+    t = (double)s + (double)c;
+  }
+  const int64_t j = idx / M, i = idx - j * M;
+  out[i * oi + j * oj] = (TO)t;
+}
+
 template <typename TP, typename TO>
 cudaError_t reduce_splits(cudaStream_t st, int64_t M, int64_t N, int nsplit, const TP* part,
                           TO* out, int64_t oi, int64_t oj) {
   const int64_t MN = M * N;
   // The flat kernel has one CTA per 1024 elements and takes the splits one after
-  // another: for an l x l Gram or the like (up to 128 x 128) the sliced one, with
-  // 32 elements a CTA, 9 -> 3 us at l = 30.  Not further: with the 64000 elements
-  // of a batch instance's T its many CTAs cost the other instances more (16 x
-  // 32768: 3090 -> 3215 us).
+  // another: for an l x l Gram or the like (up to 128 x 128) one thread per
+  // element up to 8 splits, above the sliced kernel, with 32 elements a CTA, 9 ->
+  // 3 us at l = 30.  Not further: with the 64000 elements of a batch instance's
+  // T its many CTAs cost the other instances more (16 x 32768: 3090 -> 3215 us).
   if (nsplit <= 32 && MN > 128 * 128) {
     const int vec = (sizeof(TP) == 4 && (MN & 3) == 0 && ((uintptr_t)part & 15) == 0) ? 1 : 0;
     k_reduce_flat<TP, TO><<<(unsigned)((MN + 1023) / 1024), 256, 0, st>>>(M, N, nsplit, part, out, oi,
                                                                           oj, vec);
-  }
+  } else if (nsplit <= 8)
+    k_reduce_few<TP, TO><<<(unsigned)((MN + 127) / 128), 128, 0, st>>>(M, N, nsplit, part, out, oi, oj);
   else
     k_reduce<TP, TO><<<(unsigned)((MN + 31) / 32), 256, 0, st>>>(M, N, nsplit, part, out, oi, oj);
   note_launch();
