@@ -1234,7 +1234,7 @@ constexpr size_t gated_smem_bytes(int l) {
 }
 template <typename TW>
 __global__ void __launch_bounds__(256)
-k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
+k_cholesky64_gated(int l, const double* __restrict__ G, int* gate,
                    double* __restrict__ Xout, TW* __restrict__ Xw, int ldxw, unsigned* status,
                    double* __restrict__ part, int nsplit, unsigned* ticket, double reg);
 
@@ -1374,15 +1374,18 @@ cudaError_t cholesky(cudaStream_t st, int l, const void* Gv, double tol, int rou
   }
   const size_t sm64 = gated_smem_bytes(l);
   const unsigned grid = gp && nsplit > 1 ? (unsigned)(((int64_t)l * l + 63) / 64) : 1u;
-  k_cholesky64_gated<TW><<<grid, 256, sm64, st>>>(l, nullptr, 1e-13, gate, X, Xw, ldxw, status, gp,
+  k_cholesky64_gated<TW><<<grid, 256, sm64, st>>>(l, nullptr, gate, X, Xw, ldxw, status, gp,
                                                   nsplit, status + 9, shift_coef);
   note_launch();
   return cudaGetLastError();
 }
 
+// Least share of a column's squared norm that the columns before it leave.
+constexpr double kDependent = 1e-13;
+
 template <typename TW>
 __global__ void __launch_bounds__(256)
-k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
+k_cholesky64_gated(int l, const double* __restrict__ G, int* gate,
                    double* __restrict__ Xout, TW* __restrict__ Xw, int ldxw, unsigned* status,
                    double* __restrict__ part, int nsplit, unsigned* ticket, double reg) {
   __shared__ int s_go, s_last;
@@ -1436,6 +1439,7 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
   float* Xf = (float*)sm;
   __shared__ double red[32];
   __shared__ double s_ri[kMaxL];
+  __shared__ float s_df[kMaxL];
   __shared__ int s_keep[kMaxL];
   for (int e = tid; e < l * l; e += nt) {
     const int i = e % l, j = e / l;
@@ -1443,7 +1447,10 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
     // split 0 holds the sums (written by other CTAs: read through L2)
     const double g = part ? (nsplit > 1 ? __ldcg(part + e) : part[e]) : G[e];
     A[i + j * ld] = i == j ? g + reg * g : g;
-    if (i == j) d0[j] = g;
+    if (i == j) {
+      d0[j] = g;
+      s_df[j] = (float)g;
+    }
   }
   __syncthreads();
   double dm = 0.0;
@@ -1457,7 +1464,7 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
   // other threads finish the step, so a column costs one barrier.
   const int cb = tid & 127, rg = tid >> 7, ng = nt >> 7;
   auto pivot = [&](int j, double d) {
-    const bool keep = (d0[j] > 1e-300) && (d0[j] > 1e-30 * gmax) && (d > tol * d0[j]);
+    const bool keep = (d0[j] > 1e-300) && (d0[j] > 1e-30 * gmax) && (d > kDependent * d0[j]);
     const double ri = keep ? rsqrt(d) : 0.0;
     s_keep[j] = keep ? 1 : 0;
     s_ri[j] = ri;
@@ -1512,21 +1519,28 @@ k_cholesky64_gated(int l, const double* __restrict__ G, double tol, int* gate,
     if (Xout) Xout[e] = (double)v;
     Xw[i + (int64_t)j * ldxw] = (TW)v;
   }
-  // The pivots above are those of the raised matrix, never below reg d0.  The
-  // pivot that the matrix itself has -- the squared norm left of the column
-  // after the ones before it -- is what is left of the column in Q1 = Y X,
-  // 1 - reg sum_i d0_i X_ij^2, times the raised one; a column that it shows to
-  // be dependent keeps its place (the raise completes it to a direction at
-  // rounding level) and is reported.
-  if (reg > 0.0 && tid < l && s_keep[tid]) {
-    const int j = tid;
-    double raise = 0.0;
-    for (int i = 0; i <= j; ++i) {
-      const double x = Xf[(size_t)i * ldx + j];
-      raise = fma(d0[i] * x, x, raise);
+  // R's pivots are those of the raised matrix, never below reg d0.  The pivot that
+  // the matrix itself has -- the squared norm left of a column after the ones
+  // before it -- is what is left of the column in Q1 = Y X, 1 - reg sum_i d0_i
+  // X_ij^2, times the raised one; a column that it shows to be dependent keeps its
+  // place (the raise completes it to a direction at rounding level) and is
+  // reported.  FP32 does: what is left is compared with a tenth or less, and no
+  // term of the sum is above 1.  A warp per column; a thread per column cost 18 us
+  // at l = 128.
+  if (reg > 0.0) {
+    const float rg = (float)reg;
+    for (int j = tid >> 5; j < l; j += nt >> 5) {
+      float r = 0.f;
+      for (int i = tid & 31; i < j; i += 32) {
+        const float x = Xf[(size_t)i * ldx + j];
+        r = fmaf(rg * (s_df[i] * x), x, r);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      const float xjj = rf[j], d = s_df[j] * xjj * xjj;
+      if ((tid & 31) == 0 && s_keep[j] && 1.f - (r + rg * d) <= (float)kDependent * d)
+        atomicOr(status, ST_RANK_DEF);
     }
-    const double r = 1.0 / rf[j];
-    if ((1.0 - reg * raise) * r * r <= tol * d0[j]) atomicOr(status, ST_RANK_DEF);
   }
   if (tid == 0) {
     int ndropped = 0;
