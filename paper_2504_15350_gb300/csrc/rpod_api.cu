@@ -166,10 +166,20 @@ struct Run {
 
   // D(i, c) (at D[i di + c dj]) = sum_k A(i, k) B(k, c), c < N: FP64 on the
   // SIMT pipes (split into nsplit ranges of k summed from off_part, di == 1),
-  // FP32 on the tensor cores with exactly split operands (rpod_split.cu)
+  // FP32 on the tensor cores with exactly split operands (rpod_split.cu), but
+  // for the CholeskyQR applies, fold, lift and coefficients of matrices up to 768
+  // x 768.  There the split product takes two launches (600 x 250, l = 30: 407 us a
+  // basis, 383 with the small product) and in a batch holds whole SMs: 64 instances of
+  // 400 x (100 to 200), l = 20: 1048 us, 951; l = 50: 1180 us, 1088; l = 100: 3005 us,
+  // 2919.  Larger ones take the split product, which a few rows more make the
+  // faster one at l = 128 (2000 rows: 10.9 and 11.7 us).
   int product(bool kc, int64_t M, int N, int64_t K, int nsplit, const W* A, int64_t lda, const W* B,
               int64_t ldb, W* D, int64_t di, int64_t dj, bool check) {
     if constexpr (sizeof(W) == 4) {
+      if (!kc && K <= 128 && P->n <= 768 && P->m <= 768) {
+        CK(small_product(st, M, N, (int)K, A, lda, B, ldb, D, di, dj, status, check));
+        return RPOD_OK;
+      }
       return split_gemm(st, kc, M, N, K, A, lda, B, ldb, D, di, dj, ws + P->off_planes,
                         (float*)(ws + P->off_part), P->part_elems, P->split_pct, status, check);
     } else {

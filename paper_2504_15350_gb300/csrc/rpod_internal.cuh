@@ -208,6 +208,12 @@ cudaError_t convert_snapshots(cudaStream_t st, int64_t rows, int64_t cols, const
 cudaError_t round_tf32(cudaStream_t st, int64_t rows, int64_t cols, const float* src, int64_t lds,
                        float* dst, int64_t ldd);
 
+// D[i di + c dj] = sum_k A[i + k lda] B[k + c ldb] for i < M, c < N, K <= 128, in
+// FP32 with compensated sums; check flags non-finite values of A.
+cudaError_t small_product(cudaStream_t st, int64_t M, int N, int K, const float* A, int64_t lda,
+                          const float* B, int64_t ldb, float* D, int64_t di, int64_t dj, unsigned* status,
+                          bool check);
+
 // FP64 partial Gram matrices part[z] = Y_z^T Y_z of nsplit row chunks of the
 // FP32 matrix Y (rows x l, l <= 128), products and chunk sums in FP32.
 // The same for the Gram of T^T: FP32 partials, only the upper triangle multiplied.
