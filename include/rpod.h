@@ -319,7 +319,7 @@ int rpod_batch_workspace_bytes(const rpod_batch* batch, size_t* bytes);
 int rpod_batch_run(rpod_batch* batch, void* workspace, size_t workspace_bytes, void* stream);
 /* Autotuner: times the candidate launch configurations -- worker streams in
  * {1, 2, 4, 8, 16, 32, 64} (up to the instance count) x split-K scale in
- * {1/4, 1/2, 1, 2} of the passes' default split x, for the 16-bit forms, the
+ * {1/4, 1/2, 1, 2} of the passes' default split (FP32 form: {1/4, 1/2, 1}) x, for the 16-bit forms, the
  * tensor-core passes' pipeline depth in {2, 4} stages -- as `trials` separately
  * timed replays each (CUDA events on `stream`, synchronising; a point's time
  * is the fastest replay), keeps the fastest point, re-captures, and returns
@@ -334,7 +334,9 @@ int rpod_batch_tune(rpod_batch* batch, void* workspace, size_t workspace_bytes, 
  * tuning).  Errors: RPOD_ERR_INVALID_ARG for other values. */
 int rpod_batch_set_pass_stages(rpod_batch* batch, int32_t stages);
 /* Sets the launch configuration directly (e.g. from a cached tuning):
- * 1..64 worker streams, split_pct in 10..200. */
+ * 1..64 worker streams, split_pct in 10..200 percent of the passes' default
+ * split.  The products of the FP32 form and the FP16 form's refinement pass are
+ * split for an idle GPU by default; above 100 they keep that split. */
 int rpod_batch_configure(rpod_batch* batch, int32_t streams, int32_t split_pct);
 /* Synchronises, reads and clears every instance's status word; returns the
  * first error found (and its instance index through first_bad, -1 if none)

@@ -59,7 +59,7 @@ struct rpod_plan {
   // round runs beside the refinement pass); null when they could not be made
   cudaStream_t side;
   size_t off_planes;  // FP32 form: the parts of a product's skinny operand
-  int split_pct;      // share of the default split-K of the split FP32 products
+  int split_pct;      // percentage of the default split-K of the split FP32 products (above 100: 100)
   cudaEvent_t ev_fork, ev_join;
   // graph replay of repeated basis calls: the second call with the same
   // buffers captures the launch sequence (on gcap) into gexec, later calls
@@ -762,9 +762,10 @@ static int plan_create_impl(rpod_plan** out, int64_t n, int64_t m, int32_t k, in
   P->split_pct = 100;
   if (compute != RPOD_F64) {
     // partial sums of the split FP32 products: the passes of the FP32 form,
-    // the FP16 form's refinement pass and projections
+    // the refinement pass and projections of the 16-bit ones.  Their counts
+    // are never scaled up (rpod_batch_configure).
     const size_t cap = std::max(P->part_elems, (size_t)32 << 20);
-    P->part_elems = std::max(P->part_elems, (size_t)split_count(m, n, (int)l, cap) * m * L);
+    P->part_elems = (size_t)split_count(m, n, (int)l, cap) * m * L;
     const int sy = compute == RPOD_F32 ? split_count(n, m, (int)l, cap) : 1;
     if (sy > 1) P->part_elems = std::max(P->part_elems, (size_t)sy * n * L);
   }
@@ -1403,6 +1404,7 @@ int rpod_batch_tune(rpod_batch* B, void* workspace, size_t workspace_bytes, void
   cudaStream_t st = (cudaStream_t)stream;
   const int stream_opts[7] = {1, 2, 4, 8, 16, 32, 64};
   const int split_opts[4] = {25, 50, 100, 200};
+  const int nsplit = B->compute == RPOD_F32 ? 3 : 4;  // above 100 is 100 there
   // the passes' pipeline depth matters only for the tensor-core forms
   const bool tc16 = B->compute == RPOD_BF16 || B->compute == RPOD_F16;
   const int stage_opts[2] = {2, 4};
@@ -1416,7 +1418,7 @@ int rpod_batch_tune(rpod_batch* B, void* workspace, size_t workspace_bytes, void
     if (tc16) rc = rpod_batch_set_pass_stages(B, stage_opts[g]);
     for (int a = 0; a < 7 && rc == RPOD_OK; ++a) {
       if (stream_opts[a] > std::max(1, B->count)) continue;
-      for (int b = 0; b < 4 && rc == RPOD_OK; ++b) {
+      for (int b = 0; b < nsplit && rc == RPOD_OK; ++b) {
         rc = rpod_batch_configure(B, stream_opts[a], split_opts[b]);
         if (rc == RPOD_OK) rc = rpod_batch_run(B, workspace, workspace_bytes, stream);  // capture + warm
         if (rc != RPOD_OK) break;

@@ -17,7 +17,8 @@ int split_sm_count();
 // A(i, k) = kc ? A[k + i lda] : A[i + k lda]; about as accurate as FP32
 // fused multiply-adds.  planes: split_plane_bytes(K, N) of scratch, 16-byte
 // aligned; part: part_elems floats for the partial sums (may be null); pct:
-// percentage of the default split of the k range; check flags non-finite
+// percentage of the default split of the k range, at most 100 (the default
+// is the fastest split of an idle GPU); check flags non-finite
 // values of A in *status.
 int split_gemm(cudaStream_t st, bool kc, int64_t M, int N, int64_t K, const float* A, int64_t lda,
                const float* B, int64_t ldb, float* D, int64_t di, int64_t dj, void* planes, float* part,
