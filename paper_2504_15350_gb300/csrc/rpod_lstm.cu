@@ -40,9 +40,10 @@ struct rpod_lstm {
   int64_t off_w[8][3];  // per layer: W_x, W_h, b offsets into the flat vector
   int64_t off_wy, off_by;
   // workspace layout (bytes)
-  size_t o_theta, o_m, o_v, o_grad, o_wbf, o_xtm, o_xtm2, o_gx, o_gates, o_c, o_h, o_y, o_dy,
-      o_loss, o_dhext, o_dz, o_dhrec, o_dc, o_dx, o_part, total;
-  size_t part_floats;
+  size_t o_theta, o_m, o_v, o_grad, o_wbf, o_xtm, o_xtm2, o_gates, o_c, o_h, o_y, o_loss, o_dc, total;
+  // FP32 weights only
+  size_t o_gx, o_dy, o_dhext, o_dz, o_dhrec, o_part, part_floats;
+  size_t o_xd;  // masked inputs of layers 1..L-1 (T x Bmax x H each)
   int64_t step;
   int last_launches;
   int wfp32;  // products read the FP32 master weights instead of BF16 copies
@@ -50,11 +51,10 @@ struct rpod_lstm {
   double drop_p;
   uint64_t drop_seed, drop_thr;
   int64_t drop_pass;
-  // BF16 weights: the parts of x, of every layer's h, masked h and dz, of dy
+  // BF16 weights only: the parts of x, of every layer's h, masked h and dz, of dy
   size_t o_px, o_ph, o_pxd, o_pz, o_pdy;
-  size_t o_keep;   // dropout masks of layers 1..L-1 (bytes, as o_xd)
+  size_t o_keep;   // dropout masks of layers 1..L-1 (bytes, T x Bmax x H each)
   size_t o_lpart;  // the head's shares of the loss
-  size_t o_xd;  // masked inputs of layers 1..L-1 (T x Bmax x H each)
   size_t o_bx, o_by, o_lsum;  // train_epoch: the gathered batch, the loss sum
   size_t o_sync;  // persistent rollout: barrier arrivals, abort word, status word
   // state read by rpod_lstm_load, copied to a workspace by rpod_lstm_restore
@@ -616,31 +616,32 @@ int rpod_lstm_create(rpod_lstm** out, int32_t in_dim, int32_t hidden, int32_t la
   N->o_wbf = take(2 * P);
   N->o_xtm = take(4 * T * B * I);
   N->o_xtm2 = take(4 * T * B * I);
-  N->o_gx = take(4 * layers * T * B * 4 * H);
   N->o_gates = take(4 * layers * T * B * 4 * H);
   N->o_c = take(4 * layers * (T + 1) * B * H);
   N->o_h = take(4 * layers * (T + 1) * B * H);
   N->o_y = take(4 * B * out_dim);
-  N->o_dy = take(4 * B * out_dim);
   N->o_loss = take(256);
-  N->o_dhext = take(4 * T * B * maxI);
-  N->o_dz = take(4 * T * B * 4 * H);
-  N->o_dhrec = take(4 * B * H);
-  N->o_dc = take(4 * layers * B * H);
-  N->o_dx = take(4);
-  N->part_floats = (size_t)32 * 4 * H * maxI;
-  N->o_part = take(4 * N->part_floats);
-  N->o_xd = take(4 * (size_t)(layers - 1) * T * B * H);
-  N->o_keep = take((size_t)(layers - 1) * T * B * H);
-  {
+  if (N->wfp32) {
+    N->o_gx = take(4 * layers * T * B * 4 * H);
+    N->o_dy = take(4 * B * out_dim);
+    N->o_dhext = take(4 * T * B * maxI);
+    N->o_dz = take(4 * T * B * 4 * H);
+    N->o_dhrec = take(4 * B * H);
+    N->o_dc = take(4 * B * H);
+    N->part_floats = (size_t)32 * 4 * H * maxI;
+    N->o_part = take(4 * N->part_floats);
+    N->o_xd = take(4 * (size_t)(layers - 1) * T * B * H);
+  } else {
+    N->o_dc = take(4 * layers * B * H);
+    N->o_keep = take((size_t)(layers - 1) * T * B * H);
     const size_t ldh = parts_ld(hidden), ldz = parts_ld(4 * hidden);
     N->o_px = take(6 * T * B * parts_ld(in_dim));
     N->o_ph = take(6 * layers * T * B * ldh);
     N->o_pxd = take(6 * (size_t)(layers - 1) * T * B * ldh);
     N->o_pz = take(6 * layers * T * B * ldz);
     N->o_pdy = take(6 * B * parts_ld(out_dim));
+    N->o_lpart = take(8 * (size_t)lstm_head_blocks(max_batch));
   }
-  N->o_lpart = take(8 * (size_t)lstm_head_blocks(max_batch));
   N->o_bx = take(4 * B * T * I);
   N->o_by = take(4 * B * (size_t)out_dim);
   N->o_lsum = take(4);

@@ -1,5 +1,6 @@
 """Workspace sizes (no GPU needed): the FP32 form's plans hold the partial sums that
-their products use, in a batch as alone."""
+their products use, in a batch as alone, and an LSTM the buffers of its own
+weight type."""
 import pytest
 
 import paper_2504_15350_gb300.rpod as R
@@ -35,3 +36,23 @@ def test_fp32_partials_are_those_of_its_products(n, m, k, p):
     fixed = 4 * l * (2 * n + 4 * m) + 6 * l * (n + 63) + 8 * 40 * l * l + 16 * 304 * l * l + (1 << 20)
     tiles = -(-m // 128)
     assert alone <= fixed + 4 * l * m * (2 * 152 // tiles + 2), (alone, fixed)
+
+
+@pytest.mark.parametrize("dims", [(54, 256, 2, 50, 10, 512), (14, 50, 3, 10, 10, 64), (9, 33, 1, 5, 4, 7)])
+def test_lstm_buffers_are_those_of_its_weight_type(dims):
+    I, H, L, O, T, B = dims
+    size = {}
+    for flags in (0, R.RPOD_LSTM_FP32_WEIGHTS):
+        h = R.rpod_lstm_create(*dims, flags)
+        size[flags] = R.rpod_lstm_workspace_bytes(h)
+        P = R.rpod_lstm_param_count(h)
+        R.rpod_lstm_destroy(h)
+    rows, H8, slack = T * B, (H + 7) // 8 * 8, 1 << 15
+    # parameters, moments, gradient and BF16 copy; three windows; gates, c and h
+    both = 18 * P + 12 * rows * I + 16 * L * rows * H + 8 * L * (T + 1) * B * H + 12 * B * O
+    # three BF16 parts of x, h, masked h, dz and dy, dropout masks, dc
+    bf16 = 6 * (rows * ((I + 7) // 8 * 8 + (2 * L - 1) * H8 + 4 * L * H8) + B * (O + 8)) + (L - 1) * rows * H
+    # input projections, dz, dh, masked h, split sums of the weight gradients
+    fp32 = 4 * (4 * L * rows * H + 4 * rows * H + rows * max(I, H) + (L - 1) * rows * H + 128 * H * max(I, H))
+    assert size[0] <= both + bf16 + 4 * L * B * H + slack
+    assert size[R.RPOD_LSTM_FP32_WEIGHTS] <= both + fp32 + 12 * B * max(H, O) + slack
