@@ -45,15 +45,17 @@ constexpr int kLd = 72;  // bf16 per staged row: 64 values and 16 bytes
 
 __device__ __forceinline__ float sigm_m(float x) { return 1.f / (1.f + __expf(-x)); }
 
-// a = a1 + a2 + a3 for two values, packed as bf16 pairs (low half a).  An
-// infinity is (a, 0, 0): the difference to its first part would be NaN, and
+// a = a1 + a2 + a3 for two values, packed as bf16 pairs (low half a).  INF: an
+// infinity is (a, 0, 0).  The difference to its first part would be NaN, and
 // with it every sum that the infinity alone leaves infinite (a window with an
-// infinite entry saturates its gates, as with FP32 products).
+// infinite entry saturates its gates, as with FP32 products).  Only what comes
+// from outside can be infinite while the rest stays finite: inputs and targets.
+template <bool INF>
 __device__ __forceinline__ void parts3(float a, float b, uint32_t (&p)[3]) {
   const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
   p[0] = __byte_perm(ua, ub, 0x7632);
-  const float ra = fabsf(a) == INFINITY ? 0.f : a - __uint_as_float(ua & 0xffff0000u);
-  const float rb = fabsf(b) == INFINITY ? 0.f : b - __uint_as_float(ub & 0xffff0000u);
+  const float ra = INF && fabsf(a) == INFINITY ? 0.f : a - __uint_as_float(ua & 0xffff0000u);
+  const float rb = INF && fabsf(b) == INFINITY ? 0.f : b - __uint_as_float(ub & 0xffff0000u);
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[1]) : "f"(rb), "f"(ra));
   const float qa = ra - __uint_as_float(p[1] << 16), qb = rb - __uint_as_float(p[1] & 0xffff0000u);
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[2]) : "f"(qb), "f"(qa));
@@ -199,15 +201,17 @@ __device__ __forceinline__ void stage_parts(__nv_bfloat16* dst, const Parts& P, 
   }
 }
 // the parts of a pair of neighbours (column even)
+template <bool INF = false>
 __device__ __forceinline__ void store_pair(const Parts& P, int64_t row, int col, float a, float b) {
   uint32_t w[3];
-  parts3(a, b, w);
+  parts3<INF>(a, b, w);
 #pragma unroll
   for (int q = 0; q < 3; ++q) *(uint32_t*)(P.p + q * P.plane + row * P.ld + col) = w[q];
 }
+template <bool INF = false>
 __device__ __forceinline__ void store_one(const Parts& P, int64_t row, int col, float a) {
   uint32_t w[3];
-  parts3(a, 0.f, w);
+  parts3<INF>(a, 0.f, w);
 #pragma unroll
   for (int q = 0; q < 3; ++q) *(uint16_t*)(P.p + q * P.plane + row * P.ld + col) = (uint16_t)w[q];
 }
@@ -619,7 +623,8 @@ __global__ void k_input_parts(int B, int T, int I, const float* __restrict__ X, 
   const int64_t row = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= (int64_t)T * B) return;
   const float* x = X + (row % B) * sb + (row / B) * stt;
-  for (int k = 2 * (threadIdx.x & 31); k < I; k += 64) store_pair(out, row, k, x[k], k + 1 < I ? x[k + 1] : 0.f);
+  for (int k = 2 * (threadIdx.x & 31); k < I; k += 64)
+    store_pair<true>(out, row, k, x[k], k + 1 < I ? x[k + 1] : 0.f);
 }
 
 // ---- head: a warp per batch row, lanes over the hidden units
@@ -664,7 +669,7 @@ k_head(int B, int O, int H, const float* __restrict__ h, const __nv_bfloat16* __
         y[(int64_t)b * O + o] = z;
         if (tgt) {
           const float d = z - tgt[(int64_t)b * O + o];
-          store_one(dy, b, o, 2.f / ((float)B * (float)O) * d);
+          store_one<true>(dy, b, o, 2.f / ((float)B * (float)O) * d);
           s += (double)d * d;
         }
       }
