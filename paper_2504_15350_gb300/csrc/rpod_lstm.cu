@@ -777,10 +777,11 @@ static double rollout_steps_us(const rpod_lstm* N, int B, int steps) {
   const double H = N->H, phases = N->L + N->T - 1;
   if (N->wfp32) return 25.0 + steps * (N->L * N->T * (7.0 + 0.1 * H) * (1.0 + B / 3000.0));
   const int chunks = (std::max(N->I, N->L > 1 ? N->H : 0) + 63) / 64 + (N->H + 63) / 64;
-  double us = 0.6 * chunks;  // of a phase: 16-row tiles up to 32 rows, then 64-row ones
-  if (B > 32) us = 1.3 * chunks * std::max(1.0, (B + 63) / 64 * ((N->H + 15) / 16) * std::min(N->L, N->T) / 152.0);
+  // of a phase: 16-row tiles up to 32 rows, then 64-row ones
+  double us = (B > 8 ? 3.0 : 2.0) + 0.6 * chunks;
+  if (B > 32) us = 2.5 + 1.3 * chunks * std::max(1.0, (B + 63) / 64 * ((N->H + 15) / 16) * std::min(N->L, N->T) / 152.0);
   const double odd = ((N->H | N->I) & 1) ? 1.5 : 1.0;
-  return 25.0 + steps * (8.0 + odd * phases * (2.0 + us));
+  return 25.0 + steps * (8.0 + odd * phases * us);
 }
 static double rollout_persistent_us(const rpod_lstm* N, int B, int steps, int sms) {
   const double phases = N->L + N->T - 1;
