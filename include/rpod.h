@@ -54,8 +54,9 @@ extern "C" {
  *   F32, 16-bit: Gram partials added as compensated FP32 sums, an FP32
  *                Cholesky factor with a device-gated FP64 refactorization of
  *                an exact-product Gram when a pivot shows a condition number
- *                beyond FP32 reach (F32 form: also in the second CholeskyQR
- *                round when its basis has kappa^2 > 2); the small SVD is the
+ *                beyond FP32 reach (F32 form: with the diagonal raised by
+ *                1e-12 of itself in the first round, and also in the second
+ *                when its basis has kappa^2 > 2); the small SVD is the
  *                FP32 eigen start of the Gram T T^T (FP32 products, FP64
  *                sums) refined in FP64, where eigenvalue pairs closer than
  *                the FP32 Gram's rounding level (100 u_32 ||T T^T||_F) keep
@@ -172,7 +173,9 @@ int rpod_basis(rpod_plan* plan, const void* S, int64_t lds, int32_t s_dtype,
 /* Galerkin projection of new snapshots on a basis (Sec. 4.3 coefficient
  * matrix applied to held-out data): C' = U^T S', U n x kc (kc <= l), S'
  * n x m_new.  U and C' are double for compute F64, float otherwise; S' has
- * type s_dtype as for rpod_basis.  m_new may exceed the plan's m. */
+ * type s_dtype as for rpod_basis.  m_new may exceed the plan's m.  Non-finite
+ * entries are not flagged: the coefficients that they enter are not finite (with
+ * FP32 snapshots an infinity gives NaN). */
 int rpod_project(const rpod_plan* plan, const void* U, int64_t ldu, int32_t kc,
                  const void* S_new, int64_t lds, int64_t m_new, int32_t s_dtype,
                  void* C, int64_t ldc, void* workspace, size_t workspace_bytes,
@@ -209,7 +212,8 @@ int rpod_profile_read(const rpod_plan* plan, int* passes, double* pass_ms, doubl
  * its own pool, a plugin whose execute callback may not allocate, a loop that
  * must avoid the device synchronisation an allocation can cause.  The caller
  * still passes U, S' and C' (same meaning, layout and types as rpod_project;
- * compute F64 with double data, otherwise FP32 U, S' and C').  The split-K
+ * compute F64 with double data, otherwise FP32 U, S' and C', equal to
+ * rpod_project's up to FP32 rounding).  The split-K
  * partial sums live in a 16 MiB array inside the library that every GPU which
  * loads the library holds until the process exits; nothing is allocated.
  * Limit: kc * m_new * sizeof(element) <= 16 MiB, else RPOD_ERR_UNSUPPORTED

@@ -165,10 +165,10 @@ struct Run {
   }
 
   // D(i, c) (at D[i di + c dj]) = sum_k A(i, k) B(k, c), c < N: FP64 on the
-  // SIMT pipes (split into nsplit ranges of k summed from off_part, di == 1),
-  // FP32 on the tensor cores with exactly split operands (rpod_split.cu), but
-  // for the CholeskyQR applies, fold, lift and coefficients of matrices up to 768
-  // x 768.  There the split product takes two launches (600 x 250, l = 30: 407 us a
+  // SIMT pipes (split into nsplit ranges of k summed from off_part, di == 1; the
+  // FP32 product chooses its own), FP32 on the tensor cores with operands split
+  // into bf16 parts (rpod_split.cu), but for the CholeskyQR applies, fold, lift
+  // and coefficients of matrices up to 768 x 768.  There the split product takes two launches (600 x 250, l = 30: 407 us a
   // basis, 383 with the small product) and in a batch holds whole SMs: 64 instances of
   // 400 x (100 to 200), l = 20: 1048 us, 951; l = 50: 1180 us, 1088; l = 100: 3005 us,
   // 2919.  Larger ones take the split product, which a few rows more make the
@@ -321,10 +321,12 @@ struct Run {
   // 16-bit forms: D = A B for A m x l (ld lda, a multiple of 4) and B l x N on
   // the tensor cores with exactly split operands; UNSUPPORTED leaves the product
   // to the caller.  B's parts go where the passes' 16-bit operands were (free
-  // after the last pass).  From 4096 rows on: below, the two launches take as
-  // long as the SIMT product (6 us at m = 500).  Fold and coefficients of
-  // 90225 x 85 took 74 and 43 us there; basis of 8192 x 90225: 2946 -> 2871 us,
-  // 262144 x 10000 unchanged.
+  // after the last pass).  From 4096 rows on: there the two launches take 6.3 us
+  // at l = 32, 7.1 at 64, 8.7 at 96 and 9.5 at 128, the SIMT product 5.3, 9.7, 7.6 and
+  // 9.7; at 500 rows the same within 0.2 us, at 16000 rows 6.5, 7.4, 9.1 and 9.9
+  // against 5.4, 9.9, 16.9 and 21.9.  Fold and coefficients of 90225 x 85 took
+  // 74 and 43 us on the SIMT pipes; basis of 8192 x 90225: 2946 -> 2871 us, 262144 x
+  // 10000 unchanged.
   int tall_product(int64_t M, int N, const W* A, int64_t lda, const W* B, W* D, int64_t di, int64_t dj) {
     if constexpr (sizeof(W) == 4) {
       if (is16(P->compute) && M >= 4096 && lda % 4 == 0 &&
@@ -341,8 +343,10 @@ struct Run {
     const int64_t m = P->m;
     const int l = P->l;
     // 16-bit forms: the two-part TF32 tensor-core product (about 2^-21
-    // relative error per entry, as the lift) where m is a multiple of 4, else
-    // the split product; below its size, the SIMT product
+    // relative error per entry, as the lift) where m is a multiple of 4.  At
+    // other m, where Tt1 could not be addressed by TMA before its leading
+    // dimension was rounded up, FP32's accuracy is kept: the split product, below
+    // its size the SIMT one
     int rc = RPOD_ERR_UNSUPPORTED;
     if (sizeof(W) == 4 && is16(P->compute) && m % 4 == 0)
       rc = tc_apply(st, (const float*)Tt1, ld, m, l, (const float*)buf(P->off_xw), l, (float*)out, ld,

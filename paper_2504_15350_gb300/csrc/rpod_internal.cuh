@@ -216,11 +216,11 @@ cudaError_t small_product(cudaStream_t st, int64_t M, int N, int K, const float*
 
 // FP64 partial Gram matrices part[z] = Y_z^T Y_z of nsplit row chunks of the
 // FP32 matrix Y (rows x l, l <= 128), products and chunk sums in FP32.
+cudaError_t gram_f32(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
+                     double* part);
 // The same for the Gram of T^T: FP32 partials, only the upper triangle multiplied.
 cudaError_t gram_t(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
                    float* part);
-cudaError_t gram_f32(cudaStream_t st, int64_t rows, int l, const float* Y, int64_t ldy, int nsplit,
-                     double* part);
 
 // Persistent LSTM rollout (rpod_rollout.cu): one cooperative launch for all
 // `steps` predictions; ring: the window (T x B x I, time-major), hbuf: L x T x

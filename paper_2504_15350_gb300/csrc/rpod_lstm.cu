@@ -343,8 +343,9 @@ struct Net {
 
   // y (B x O) of the input X (element (b, t, k) at X[b sb + t stt + k]); with a
   // target also dy and (FP32 weights) the loss.  Xt: the time-major input of
-  // the FP32-weight kernels, made from X unless X has that layout itself.  BF16 weights: tensor-core cells, one launch per
-  // anti-diagonal (rpod_lstm_mma.cu); FP32 weights: the SIMT kernels here.
+  // the FP32-weight kernels, made from X unless X has that layout itself.
+  // BF16 weights: tensor-core cells, one launch per anti-diagonal
+  // (rpod_lstm_mma.cu); FP32 weights: the SIMT kernels here.
   int forward(const float* X, int64_t sb, int64_t stt, float* Xt, int B, float* y, const float* tgt) {
     if (!N->wfp32) {
       LK(lstm_input_parts(st, B, N->T, N->I, X, sb, stt, px()));

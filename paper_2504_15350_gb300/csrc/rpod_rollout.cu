@@ -1,5 +1,7 @@
-// Persistent LSTM rollout (the online stage of Sec. 4.3): autoregressive
-// prediction of `steps` coefficient vectors in one cooperative launch.
+// LSTM rollout kernels (the online stage of Sec. 4.3): autoregressive
+// prediction of `steps` coefficient vectors in one launch.  The pipelined kernel
+// over a cluster per sample is the second half of this file; first the
+// persistent cooperative kernel, for what it does not fit or takes longer for.
 //
 // The network maps a window of T rows [mu, alpha] to the next alpha, with
 // zero initial states for every window, so each prediction runs L x T cells.
@@ -283,13 +285,16 @@ __global__ void __launch_bounds__(512, 1) k_rollout(RollArgs a) {
 // weight load and T/4 broadcast 16-byte loads of h for T packed FMAs.  New h
 // values go to every CTA of the cluster as bulk copies between shared memories
 // that complete on the receiver's mbarrier; the wait for them comes after the
-// next phase's recurrent product, which needs only the previous row.  The head is split over the units: each CTA sends its share of
-// the O outputs with its h, and every CTA adds the CS shares itself.
+// next phase's recurrent product, which needs only the previous row.  The head
+// is split over the units: each CTA sends its share of the O outputs with its
+// h, and every CTA adds the CS shares itself.
 //
 // Bound: the FP32 pipes (3 products of 4U x T x H per row and CTA) and the
 // phase latency (partial sums over the k-slices, gates, exchange).  Measured
 // at 2 x 256, window 10, 8 samples, 500 steps: 4.1 ms; the kernel with
-// T + L - 1 grid barriers per prediction above takes 68.4 ms.
+// T + L - 1 grid barriers per prediction above takes 68.4 ms.  Every wave of
+// clusters loads the weights and runs the window first, so many samples over
+// few steps take the per-step kernels (rollout_pipelined's limit).
 constexpr int kPipeThreads = 384;
 constexpr size_t kPipeSmemMax = (size_t)226 * 1024;
 

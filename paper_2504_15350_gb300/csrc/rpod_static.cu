@@ -1,7 +1,9 @@
 // Allocation-free Galerkin projection (C' = U^T S', the coefficients of new
-// snapshots on the basis, Sec. 4.3): the rpod_project computation with its
-// split-K partial sums kept in a fixed device array of this library instead
-// of a caller-provided workspace.
+// snapshots on the basis, Sec. 4.3): rpod_project's product with its split-K
+// partial sums kept in a fixed device array of this library instead of a
+// caller-provided workspace.  FP32 snapshots are multiplied by FP32 FMAs here,
+// in three bf16 parts on the tensor cores there (which needs room for the
+// parts of U), so the two differ in rounding, and this one takes longer.
 //
 // Some callers cannot call cudaMalloc or hand out a workspace: a host
 // framework that owns every byte of device memory through its own pool, a

@@ -206,7 +206,7 @@ def rpod_sample(plan, A, lda, S, lds, s_dtype, Y, ldy, ws, ws_bytes, stream):
 
 
 def rpod_project_static(plan, U, ldu, kc, S_new, lds, m_new, s_dtype, C, ldc, stream):
-    """Allocation-free projection: same result as rpod_project, with the
+    """Allocation-free projection: rpod_project (up to FP32 rounding) with the
     split-K scratch in a fixed 16 MiB device array of the library (for
     callers that cannot allocate device memory or hand out a workspace)."""
     return load().rpod_project_static(plan, U, ldu, kc, S_new, lds, m_new, s_dtype, C, ldc, stream)
